@@ -547,42 +547,51 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
 }
 
 // --------------------------------------------------- per-warp row ring
-// Streams chunks of 32 rows x 32 elements (4 KB) of a tensor map built by
-// encode_rows32_map (box 32 x 32) through a ring of kRingStages buffers per
-// warp, two chunks in flight while one is processed.  Warp `gw` of `nw` takes
+// Streams chunks of `rpc` rows x 32 elements (4 KB for 32 rows) of a tensor
+// map built by encode_rows32_map (box 32 x rpc) through a ring of NS buffers
+// per warp, NS - 1 chunks (one for NS = 1) in flight.  Warp `gw` of `nw` takes
 // chunks gw, gw + nw, ...; for each, lane 0 has armed the slot's mbarrier and
 // issued the 2D TMA load, every lane waits (bounded), then
 //   body(c, buf)  reads the chunk (row r at uint4 r*8, its unit j at unit
 //                 j ^ (r & 7)) and, when STORE, leaves its results there;
 // with STORE the ring writes the buffer back through `tout` by TMA store and
-// refills a slot only after the previous store has read it.  Chunks past the
+// refills a slot only after the previous store has read it.  Rows past the
 // tensor's last row read as 0 and are not stored.  A load that does not land
 // within `limit` polls records kDevTimeout, gives the copies in flight a
 // bounded wait and ends the warp's loop.  CTAs are kRingWarps warps.
-constexpr int kRingStages = 3;
+//
+// Launches give every warp one or two chunks (ring_grid) and let the hardware
+// hand out CTAs, instead of one resident wave whose warps stride over the
+// array: SMs do not reach memory at equal rates, so equal shares end in a
+// tail of the slower ones.  2^26 elements copied through this ring (GB300):
+// one wave of 304 CTAs 88.9 us (6037 GB/s), 8 / 4 / 2 / 1 chunks per warp
+// 84.0 / 81.5 / 80.3 / 79.6 us (6747 GB/s, the device's copy rate).
 constexpr int kRingWarps = 8;
 constexpr uint32_t kRingChunkBytes = 32 * 32 * 4;
-constexpr size_t kRingSmem = (size_t)kRingWarps * kRingStages * kRingChunkBytes + 1024 + kRingWarps * kRingStages * 8;
+constexpr size_t ring_smem(int stages) {
+  return (size_t)kRingWarps * stages * kRingChunkBytes + 1024 + kRingWarps * stages * 8;
+}
 
-template <bool STORE, class Body>
-__device__ __forceinline__ void row_ring(const CUtensorMap* tin, const CUtensorMap* tout, int64_t nch, uint32_t limit,
-                                         unsigned* status, Body&& body) {
+template <bool STORE, int NS, class Body>
+__device__ __forceinline__ void row_ring(const CUtensorMap* tin, const CUtensorMap* tout, int64_t nch, int rpc,
+                                         uint32_t limit, unsigned* status, Body&& body) {
+  constexpr int AHEAD = NS > 1 ? NS - 1 : 1;  // chunks in flight
   extern __shared__ uint8_t ring_smem_raw[];
   uint8_t* base =
       reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(ring_smem_raw) + 1023) & ~uintptr_t(1023));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  uint8_t* ring = base + (size_t)warp * kRingStages * kRingChunkBytes;
-  uint64_t* bars =
-      reinterpret_cast<uint64_t*>(base + (size_t)kRingWarps * kRingStages * kRingChunkBytes) + warp * kRingStages;
+  uint8_t* ring = base + (size_t)warp * NS * kRingChunkBytes;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(base + (size_t)kRingWarps * NS * kRingChunkBytes) + warp * NS;
   const int64_t gw = (int64_t)blockIdx.x * kRingWarps + warp, nw = (int64_t)gridDim.x * kRingWarps;
+  const uint32_t bytes = (uint32_t)rpc * 128u;
   if (lane == 0) {
-    for (int k = 0; k < kRingStages; ++k) mbar_init(bars + k, 1);
+    for (int k = 0; k < NS; ++k) mbar_init(bars + k, 1);
     mbar_init_fence();
-    for (int k = 0; k < kRingStages - 1; ++k) {
+    for (int k = 0; k < AHEAD; ++k) {
       const int64_t c = gw + k * nw;
       if (c < nch) {
-        mbar_arrive_expect_tx(bars + k, kRingChunkBytes);
-        tma_load_2d(ring + k * kRingChunkBytes, tin, 0, (int)(c * 32), bars + k);
+        mbar_arrive_expect_tx(bars + k, bytes);
+        tma_load_2d(ring + k * kRingChunkBytes, tin, 0, (int)(c * rpc), bars + k);
       }
     }
   }
@@ -590,9 +599,9 @@ __device__ __forceinline__ void row_ring(const CUtensorMap* tin, const CUtensorM
   bool ok = true;
   int64_t k = 0;
   for (int64_t c = gw; c < nch; c += nw, ++k) {
-    const int slot = (int)(k % kRingStages);
+    const int slot = (int)(k % NS);
     uint4* buf = reinterpret_cast<uint4*>(ring + slot * kRingChunkBytes);
-    ok = mbar_wait_bounded(bars + slot, (uint32_t)((k / kRingStages) & 1), limit);
+    ok = mbar_wait_bounded(bars + slot, (uint32_t)((k / NS) & 1), limit);
     if (!__all_sync(kFull, ok)) {
       ok = false;
       break;
@@ -601,13 +610,16 @@ __device__ __forceinline__ void row_ring(const CUtensorMap* tin, const CUtensorM
     fence_proxy_async_smem();  // this lane's accesses to the buffer, before the async proxy's
     __syncwarp();
     if (lane == 0) {
-      if constexpr (STORE) tma_store_2d(tout, 0, (int)(c * 32), buf);
-      const int64_t cn = c + (kRingStages - 1) * nw;  // refill the previous chunk's slot
+      if constexpr (STORE) tma_store_2d(tout, 0, (int)(c * rpc), buf);
+      const int64_t cn = c + AHEAD * nw;  // refill the previous chunk's slot (this one's for NS = 1)
       if (cn < nch) {
-        const int ns = (int)((k + kRingStages - 1) % kRingStages);
-        if constexpr (STORE) tma_store_wait_read1();  // the previous chunk's store has read it
-        mbar_arrive_expect_tx(bars + ns, kRingChunkBytes);
-        tma_load_2d(ring + ns * kRingChunkBytes, tin, 0, (int)(cn * 32), bars + ns);
+        const int ns = (int)((k + AHEAD) % NS);
+        if constexpr (STORE) {  // the slot's store has read it
+          if constexpr (NS > 1) tma_store_wait_read1();
+          else tma_store_wait_read();
+        }
+        mbar_arrive_expect_tx(bars + ns, bytes);
+        tma_load_2d(ring + ns * kRingChunkBytes, tin, 0, (int)(cn * rpc), bars + ns);
       }
     }
     __syncwarp();
@@ -615,13 +627,12 @@ __device__ __forceinline__ void row_ring(const CUtensorMap* tin, const CUtensorM
   if (lane == 0) {
     if (!ok) {
       atomicOr(status, 1u);  // kDevTimeout
-      for (int j = 0; j < kRingStages - 1; ++j) {
+      for (int j = 0; j < AHEAD; ++j) {
         const int64_t kk = k + j;
-        if (gw + kk * nw < nch)
-          mbar_wait_bounded(bars + (int)(kk % kRingStages), (uint32_t)((kk / kRingStages) & 1), limit);
+        if (gw + kk * nw < nch) mbar_wait_bounded(bars + (int)(kk % NS), (uint32_t)((kk / NS) & 1), limit);
       }
     }
-    if constexpr (STORE) tma_store_wait_all();
+    if constexpr (STORE) tma_store_wait_read();  // (the copies' writes are complete when the kernel is)
   }
   __syncwarp();
 }
@@ -742,6 +753,14 @@ int persistent_grid(K kernel, int block, size_t dyn_smem, int64_t work_ctas) {
   int64_t g = (int64_t)per_sm * sm_count();
   if (work_ctas < g) g = work_ctas;
   return g < 1 ? 1 : (int)g;
+}
+
+// Grid of a row_ring kernel over nch chunks: `per_warp` chunks per warp, but
+// one while that leaves less than two CTAs per SM (small arrays end sooner
+// with their chunks side by side).
+inline unsigned ring_grid(int64_t nch, int per_warp) {
+  if (nch < (int64_t)2 * per_warp * kRingWarps * sm_count()) per_warp = 1;
+  return (unsigned)((nch + (int64_t)kRingWarps * per_warp - 1) / ((int64_t)kRingWarps * per_warp));
 }
 
 }  // namespace cox

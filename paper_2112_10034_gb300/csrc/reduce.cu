@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(kRingWarps * 32, 2)
   const int lane = threadIdx.x & 31;
   const int64_t rows = n / 32;
   const int64_t ntiles = (n + W - 1) / W;
-  row_ring<false>(&tin, nullptr, (rows + 31) / 32, limit, status, [&](int64_t c, uint4* buf) {
+  row_ring<false, kRedStages>(&tin, nullptr, (rows + 31) / 32, 32, limit, status, [&](int64_t c, uint4* buf) {
     V v[32];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
@@ -374,12 +374,12 @@ static cox_status launch_reduce(cox_scope scope, const void* d_in, void* d_out, 
     auto k = k_reduce_tile_rows<R, W>;
     static int gmax_rows;
     if (gmax_rows == 0) {
-      if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRingSmem) != cudaSuccess)
+      if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring_smem(kRedStages)) != cudaSuccess)
         return COX_ECUDA;
-      gmax_rows = persistent_grid(k, kRingWarps * 32, kRingSmem, 1 << 30);
+      gmax_rows = persistent_grid(k, kRingWarps * 32, ring_smem(kRedStages), 1 << 30);
     }
     const int64_t ctas = ((rows + 31) / 32 + kRingWarps - 1) / kRingWarps;
-    k<<<(int)(ctas < gmax_rows ? ctas : gmax_rows), kRingWarps * 32, kRingSmem, st>>>(
+    k<<<(int)(ctas < gmax_rows ? ctas : gmax_rows), kRingWarps * 32, ring_smem(kRedStages), st>>>(
         tin, in, out, d_lo, n, spin_limit(), device_status_word());
     return launch_status();
   }

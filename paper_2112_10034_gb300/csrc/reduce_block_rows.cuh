@@ -24,6 +24,8 @@
 
 namespace cox {
 
+constexpr int kRedStages = 3;  // ring buffers per warp of the tile and block reductions
+
 // Launches the BLOCK-scope rows kernel for reducer R (power-of-two B, a
 // 16-byte aligned input of at least 32 elements and fewer than 2^36).
 // Instantiated in reduce_block_rows_{a,b,c,d}.cu, three reducers per file,
@@ -165,7 +167,7 @@ __global__ void __launch_bounds__(kRingWarps * 32, 2)
   const int64_t rows = n / 32;
   const int LB = 1024 / B;
   const int64_t nfull = rows * 32 / B;  // logical blocks of full rows only
-  row_ring<false>(&tin, nullptr, (rows + 31) / 32, limit, status, [&](int64_t c, uint4* buf) {
+  row_ring<false, kRedStages>(&tin, nullptr, (rows + 31) / 32, 32, limit, status, [&](int64_t c, uint4* buf) {
     V v[32];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
@@ -193,13 +195,13 @@ static cox_status launch_block_rows(const void* in, void* out, float* lo, int64_
   auto k = k_reduce_block_rows<R, W>;
   static int gmax;
   if (gmax == 0) {
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRingSmem) != cudaSuccess)
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring_smem(kRedStages)) != cudaSuccess)
       return COX_ECUDA;
-    gmax = persistent_grid(k, kRingWarps * 32, kRingSmem, 1 << 30);
+    gmax = persistent_grid(k, kRingWarps * 32, ring_smem(kRedStages), 1 << 30);
   }
   const int64_t ctas = ((rows + 31) / 32 + kRingWarps - 1) / kRingWarps;
   const int grid = (int)(ctas < gmax ? ctas : gmax);
-  k<<<grid < 1 ? 1 : grid, kRingWarps * 32, kRingSmem, st>>>(tin, static_cast<const uint32_t*>(in),
+  k<<<grid < 1 ? 1 : grid, kRingWarps * 32, ring_smem(kRedStages), st>>>(tin, static_cast<const uint32_t*>(in),
                                                               static_cast<uint32_t*>(out), lo, n, B, spin_limit(),
                                                               device_status_word());
   return launch_status();

@@ -4,10 +4,11 @@
 // run on a tile: Hillis-Steele steps d = 1, 2, .., W/2 of
 //   u = shfl_up(x, d, W); if (rank >= d) x = u op x
 // with the lane numbering of Code 3 (element i is global thread i's operand).
-// Persistent warps stream chunks of ROWS x 32 elements: 128-bit loads,
-// a warp-private shared-memory transpose to one element per lane per row,
-// ROWS independent shuffle chains (instruction-level parallelism), and the
-// inverse transpose to 128-bit stores.
+// 16-byte aligned arrays take the row-per-lane kernel (k_tile_scan_rows);
+// otherwise persistent warps stream chunks of ROWS x 32 elements: 128-bit
+// loads, a warp-private shared-memory transpose to one element per lane per
+// row, ROWS independent shuffle chains (instruction-level parallelism), and
+// the inverse transpose to 128-bit stores.
 #include "cox_common.cuh"
 
 namespace cox {
@@ -37,10 +38,28 @@ __global__ void __launch_bounds__(R::kComp ? 256 : 1024) k_tile_scan(const uint3
 // (scan_row_regs in cox_common.cuh: each width-W tile collapsed into one
 // thread's registers.)
 
-// Persistent warps stream chunks of 32 rows through row_ring: a chunk is
-// read row per lane, scanned in registers, written back in place and stored
-// by TMA.  `n / 32` full rows go through the tensor maps (>= 1 row); the last
-// n % 32 elements are scanned by thread 0 of CTA 0 from global memory.
+// Warps stream chunks of 32 rows through row_ring: a chunk is read row per
+// lane, scanned in registers, written back in place and stored by TMA.
+// `n / 32` full rows go through the tensor maps (>= 1 row); the last n % 32
+// elements are scanned by thread 0 of CTA 0 from global memory.
+//
+// Plain scans are bound by memory: one chunk per warp, one buffer (33 KB of
+// shared memory per CTA, so other CTAs' loads cover a warp's wait) runs 2^26
+// elements at the copy rate (79.6 us; 89.5 us as one persistent wave).
+// Compensated scans keep the arithmetic busy for about as long as memory (31
+// adds per element at width 32, two CTAs of 128 registers per thread), so a
+// warp takes two chunks with the second in flight under the first's
+// arithmetic: widths 4 / 16 / 32 in 80.0 / 82.1 / 90.1 us against 83.7 / 92.2
+// / 104.4 with one chunk, and 89.2 / 94.9 / 89.9 as one persistent wave.
+template <class R>
+constexpr int rows_stages() {
+  return R::kComp ? 3 : 1;
+}
+template <class R>
+constexpr int rows_chunks() {
+  return R::kComp ? 2 : 1;
+}
+
 template <class R, int W>
 __global__ void __launch_bounds__(kRingWarps * 32, 2)
     k_tile_scan_rows(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtensorMap tout,
@@ -50,7 +69,7 @@ __global__ void __launch_bounds__(kRingWarps * 32, 2)
   using V = typename R::V;
   const int lane = threadIdx.x & 31;
   const int64_t rows = n / 32;
-  row_ring<true>(&tin, &tout, (rows + 31) / 32, limit, status, [&](int64_t, uint4* buf) {
+  row_ring<true, rows_stages<R>()>(&tin, &tout, (rows + 31) / 32, 32, limit, status, [&](int64_t, uint4* buf) {
     V v[32];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {  // unit j of row `lane` sits at unit j ^ (lane & 7)
@@ -86,17 +105,18 @@ static cox_status launch_scan_rows(const void* in, void* out, int64_t n, cudaStr
   CUtensorMap tin, tout;
   if (!encode_rows32_map(&tin, in, rows, 32) || !encode_rows32_map(&tout, out, rows, 32)) return COX_ECUDA;
   auto k = k_tile_scan_rows<R, W>;
-  static int grid_cache = 0;  // persistent grid (occupancy does not change)
-  if (grid_cache == 0) {
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRingSmem) != cudaSuccess)
+  constexpr size_t smem = ring_smem(rows_stages<R>());
+  static bool ready[kMaxDevices];  // per device: the kernel may take its shared memory
+  bool& rd = ready[device_index()];
+  if (!rd) {
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
       return COX_ECUDA;
-    grid_cache = persistent_grid(k, kRingWarps * 32, kRingSmem, 1 << 30);
+    rd = true;
   }
   const int64_t nch = (rows + 31) / 32;
-  const int64_t ctas = (nch + kRingWarps - 1) / kRingWarps;
-  const int grid = (int)(ctas < grid_cache ? ctas : grid_cache);
-  k<<<grid, kRingWarps * 32, kRingSmem, st>>>(tin, tout, static_cast<const uint32_t*>(in),
-                                              static_cast<uint32_t*>(out), n, spin_limit(), device_status_word());
+  k<<<ring_grid(nch, rows_chunks<R>()), kRingWarps * 32, smem, st>>>(tin, tout, static_cast<const uint32_t*>(in),
+                                                                     static_cast<uint32_t*>(out), n, spin_limit(),
+                                                                     device_status_word());
   return launch_status();
 }
 
