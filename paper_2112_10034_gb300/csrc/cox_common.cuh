@@ -659,6 +659,94 @@ __device__ __forceinline__ void scan_row_regs(typename R::V (&v)[32]) {
   }
 }
 
+// Two fp32 values in a 64-bit register pair: one add.rn.f32x2 adds both, each
+// rounded as __fadd_rn rounds it.
+__device__ __forceinline__ uint64_t f2_pack(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void f2_unpack(uint64_t p, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(p));
+}
+__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t f2_sub(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ void f2_two_sum(uint64_t a, uint64_t b, uint64_t& s, uint64_t& t) {
+  s = f2_add(a, b);
+  const uint64_t bp = f2_sub(s, a);
+  const uint64_t ap = f2_sub(s, bp);
+  t = f2_add(f2_sub(a, ap), f2_sub(b, bp));
+}
+
+// The compensated row on packed pairs: s[k] and e[k] end as the sum and error
+// words of elements 2k and 2k + 1.  From distance 2 on both operands of a
+// step are aligned pairs, so two combines take one combine's instructions
+// (at width 32, 15.7 packed adds per element instead of 31.3): the
+// compensated scans are bound by issue, not by the adders' rate.
+template <int W>
+__device__ __forceinline__ void scan_row_pairs(const float (&x)[32], uint64_t (&s)[16], uint64_t (&e)[16]) {
+  constexpr int P = W / 2;  // pairs per tile
+#pragma unroll
+  for (int k0 = 0; k0 < 16; k0 += P) {
+#pragma unroll
+    for (int k = k0; k < k0 + P; ++k) {  // d = 1, on fresh values (error words zero)
+      const float x0 = x[2 * k], x1 = x[2 * k + 1];
+      f2_two_sum(f2_pack(k > k0 ? x[2 * k - 1] : 0.0f, x0), f2_pack(x0, x1), s[k], e[k]);
+      if (k == k0) {  // the tile's first element has no left neighbour
+        float lo, hi;
+        f2_unpack(s[k], lo, hi);
+        s[k] = f2_pack(x0, hi);
+        f2_unpack(e[k], lo, hi);
+        e[k] = f2_pack(0.0f, hi);
+      }
+    }
+#pragma unroll
+    for (int d = 1; d < P; d <<= 1)
+#pragma unroll
+      for (int k = k0 + P - 1; k >= k0 + d; --k) {
+        uint64_t ns, t;
+        f2_two_sum(s[k - d], s[k], ns, t);
+        s[k] = ns;
+        e[k] = f2_add(f2_add(e[k - d], e[k]), t);
+      }
+  }
+}
+
+// Scans the tiles of one row in place, element bits in, result bits out.
+template <class R, int W>
+__device__ __forceinline__ void scan_row(uint32_t (&w)[32]) {
+  using T = typename R::T;
+  if constexpr (R::kComp) {
+    float x[32];
+    uint64_t s[16], e[16];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) x[i] = __uint_as_float(w[i]);
+    scan_row_pairs<W>(x, s, e);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      float lo, hi;
+      f2_unpack(f2_add(s[k], e[k]), lo, hi);
+      w[2 * k] = __float_as_uint(lo);
+      w[2 * k + 1] = __float_as_uint(hi);
+    }
+  } else {
+    typename R::V v[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) v[i] = R::load(from_bits<T>(w[i]));
+    scan_row_regs<R, W>(v);
+#pragma unroll
+    for (int i = 0; i < 32; ++i) w[i] = to_bits(R::out(v[i]));
+  }
+}
+
 // ------------------------------------------------------------ host helpers
 // The driver's tensor-map encoder (looked up once; null if unavailable).
 inline PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {

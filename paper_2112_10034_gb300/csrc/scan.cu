@@ -35,7 +35,7 @@ __global__ void __launch_bounds__(R::kComp ? 256 : 1024) k_tile_scan(const uint3
 }
 
 // ------------------------------------------------ one tile row per lane
-// (scan_row_regs in cox_common.cuh: each width-W tile collapsed into one
+// (scan_row in cox_common.cuh: each width-W tile collapsed into one
 // thread's registers.)
 
 // Warps stream chunks of 32 rows through row_ring: a chunk is read row per
@@ -46,11 +46,12 @@ __global__ void __launch_bounds__(R::kComp ? 256 : 1024) k_tile_scan(const uint3
 // Plain scans are bound by memory: one chunk per warp, one buffer (33 KB of
 // shared memory per CTA, so other CTAs' loads cover a warp's wait) runs 2^26
 // elements at the copy rate (79.6 us; 89.5 us as one persistent wave).
-// Compensated scans keep the arithmetic busy for about as long as memory (31
+// Compensated scans keep the arithmetic busy for most of that time (16 packed
 // adds per element at width 32, two CTAs of 128 registers per thread), so a
 // warp takes two chunks with the second in flight under the first's
-// arithmetic: widths 4 / 16 / 32 in 80.0 / 82.1 / 90.1 us against 83.7 / 92.2
-// / 104.4 with one chunk, and 89.2 / 94.9 / 89.9 as one persistent wave.
+// arithmetic: widths 4 / 16 / 32 in 79.9 / 80.0 / 81.7 us, against 80.0 /
+// 87.8 / 94.5 with one chunk, 80.0 / 82.1 / 90.1 with unpacked adds, and 89.2
+// / 94.9 / 89.9 as one persistent wave with unpacked adds.
 template <class R>
 constexpr int rows_stages() {
   return R::kComp ? 3 : 1;
@@ -65,37 +66,34 @@ __global__ void __launch_bounds__(kRingWarps * 32, 2)
     k_tile_scan_rows(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtensorMap tout,
                      const uint32_t* __restrict__ in, uint32_t* __restrict__ out, int64_t n, uint32_t limit,
                      unsigned* status) {
-  using T = typename R::T;
-  using V = typename R::V;
   const int lane = threadIdx.x & 31;
   const int64_t rows = n / 32;
   row_ring<true, rows_stages<R>()>(&tin, &tout, (rows + 31) / 32, 32, limit, status, [&](int64_t, uint4* buf) {
-    V v[32];
+    uint32_t w[32];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {  // unit j of row `lane` sits at unit j ^ (lane & 7)
       const uint4 q = buf[lane * 8 + (j ^ (lane & 7))];
-      v[4 * j] = R::load(from_bits<T>(q.x));
-      v[4 * j + 1] = R::load(from_bits<T>(q.y));
-      v[4 * j + 2] = R::load(from_bits<T>(q.z));
-      v[4 * j + 3] = R::load(from_bits<T>(q.w));
+      w[4 * j] = q.x;
+      w[4 * j + 1] = q.y;
+      w[4 * j + 2] = q.z;
+      w[4 * j + 3] = q.w;
     }
-    scan_row_regs<R, W>(v);
+    scan_row<R, W>(w);
 #pragma unroll
     for (int j = 0; j < 8; ++j)
-      buf[lane * 8 + (j ^ (lane & 7))] = make_uint4(to_bits(R::out(v[4 * j])), to_bits(R::out(v[4 * j + 1])),
-                                                    to_bits(R::out(v[4 * j + 2])), to_bits(R::out(v[4 * j + 3])));
+      buf[lane * 8 + (j ^ (lane & 7))] = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
   });
   // The last n % 32 elements: one lane, padded.
   if (blockIdx.x == 0 && threadIdx.x == 0 && rows * 32 < n) {
     const int64_t b = rows * 32;
     const int m = (int)(n - b);
-    V v[32];
+    uint32_t w[32];
 #pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = R::load(i < m ? from_bits<T>(in[b + i]) : R::pad());
-    scan_row_regs<R, W>(v);
+    for (int i = 0; i < 32; ++i) w[i] = i < m ? in[b + i] : to_bits(R::pad());
+    scan_row<R, W>(w);
 #pragma unroll
     for (int i = 0; i < 32; ++i)
-      if (i < m) out[b + i] = to_bits(R::out(v[i]));
+      if (i < m) out[b + i] = w[i];
   }
 }
 

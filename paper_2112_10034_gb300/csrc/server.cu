@@ -202,32 +202,28 @@ __global__ void __launch_bounds__(kServeBlock) k_serve_reduce_solo(const ReqDesc
 // ------------------------------------------------------------------ scan
 // Thread t scans rows t and t + 256 of the tile (row r = elements 32 r ..
 // 32 r + 31) in registers, each width-W tile collapsed into the thread
-// (scan_row_regs), in place.  The tile is linear in shared memory (one 1D
+// (scan_row), in place.  The tile is linear in shared memory (one 1D
 // bulk copy per request tile), so a lane's 16-byte reads of its row meet
 // 8-way bank conflicts; the tile's arithmetic, not shared memory, bounds it.
 template <class R, int W>
 __device__ void serve_scan_rows(uint32_t* buf, int rows) {
-  using T = typename R::T;
-  using V = typename R::V;
   uint4* b4 = reinterpret_cast<uint4*>(buf);
 #pragma unroll 1
   for (int h = 0; h < (int)(kTile / 32 / kServeBlock); ++h) {
     const int r = h * kServeBlock + threadIdx.x;
     if (r >= rows) break;  // rows past a partial tile's end are not needed
-    V v[32];
+    uint32_t w[32];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const uint4 q = b4[r * 8 + j];
-      v[4 * j] = R::load(from_bits<T>(q.x));
-      v[4 * j + 1] = R::load(from_bits<T>(q.y));
-      v[4 * j + 2] = R::load(from_bits<T>(q.z));
-      v[4 * j + 3] = R::load(from_bits<T>(q.w));
+      w[4 * j] = q.x;
+      w[4 * j + 1] = q.y;
+      w[4 * j + 2] = q.z;
+      w[4 * j + 3] = q.w;
     }
-    scan_row_regs<R, W>(v);
+    scan_row<R, W>(w);
 #pragma unroll
-    for (int j = 0; j < 8; ++j)
-      b4[r * 8 + j] = make_uint4(to_bits(R::out(v[4 * j])), to_bits(R::out(v[4 * j + 1])),
-                                 to_bits(R::out(v[4 * j + 2])), to_bits(R::out(v[4 * j + 3])));
+    for (int j = 0; j < 8; ++j) b4[r * 8 + j] = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
   }
 }
 

@@ -19,8 +19,8 @@ def test_compensated_tile_scan_around_two_chunks_per_warp(cox, delta):  # noqa: 
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     n = 4 * WARPS * sms * CHUNK + delta
     x = inputs.normal_f32(n, seed=7)
-    out = poisoned(n, torch.float32)
-    assert cox.cox_tile_scan(o.SUM, o.F32, 16, 256, dev(x).data_ptr(), out.data_ptr(), n, 1, None) == cox.COX_OK
+    xd, out = dev(x), poisoned(n, torch.float32)
+    assert cox.cox_tile_scan(o.SUM, o.F32, 16, 256, xd.data_ptr(), out.data_ptr(), n, 1, None) == cox.COX_OK
     got = host(out)
     assert (got[n:].view(np.int32) == POISON).all()
     want = o.scan_emulate(o.SUM, o.F32, 16, 256, x, compensated=True)
