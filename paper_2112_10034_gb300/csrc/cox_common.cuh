@@ -556,7 +556,7 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
 //                 j ^ (r & 7)) and, when STORE, leaves its results there;
 // with STORE the ring writes the buffer back through `tout` by TMA store and
 // refills a slot only after the previous store has read it.  Rows past the
-// tensor's last row read as 0 and are not stored.  A load that does not land
+// tensor's last row (`rows`) read as 0 and are not stored.  A load that does not land
 // within `limit` polls records kDevTimeout, gives the copies in flight a
 // bounded wait and ends the warp's loop.  CTAs are kRingWarps warps.
 //
@@ -573,8 +573,8 @@ constexpr size_t ring_smem(int stages) {
 }
 
 template <bool STORE, int NS, class Body>
-__device__ __forceinline__ void row_ring(const CUtensorMap* tin, const CUtensorMap* tout, int64_t nch, int rpc,
-                                         uint32_t limit, unsigned* status, Body&& body) {
+__device__ __forceinline__ void row_ring(const CUtensorMap* tin, const CUtensorMap* tout, int64_t rows, int64_t nch,
+                                         int rpc, uint32_t limit, unsigned* status, Body&& body) {
   constexpr int AHEAD = NS > 1 ? NS - 1 : 1;  // chunks in flight
   extern __shared__ uint8_t ring_smem_raw[];
   uint8_t* base =
@@ -610,7 +610,8 @@ __device__ __forceinline__ void row_ring(const CUtensorMap* tin, const CUtensorM
     fence_proxy_async_smem();  // this lane's accesses to the buffer, before the async proxy's
     __syncwarp();
     if (lane == 0) {
-      if constexpr (STORE) tma_store_2d(tout, 0, (int)(c * rpc), buf);
+      if constexpr (STORE)
+        if (c * rpc < rows) tma_store_2d(tout, 0, (int)(c * rpc), buf);
       const int64_t cn = c + AHEAD * nw;  // refill the previous chunk's slot (this one's for NS = 1)
       if (cn < nch) {
         const int ns = (int)((k + AHEAD) % NS);

@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(kRingWarps * 32, 2)
   const int lane = threadIdx.x & 31;
   const int64_t rows = n / 32;
   const int64_t ntiles = (n + W - 1) / W;
-  row_ring<false, kRedStages>(&tin, nullptr, (rows + 31) / 32, 32, limit, status, [&](int64_t c, uint4* buf) {
+  row_ring<false, kRedStages>(&tin, nullptr, rows, (rows + 31) / 32, 32, limit, status, [&](int64_t c, uint4* buf) {
     V v[32];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {

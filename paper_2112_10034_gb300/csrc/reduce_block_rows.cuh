@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(kRingWarps * 32, 2)
   const int64_t rows = n / 32;
   const int LB = 1024 / B;
   const int64_t nfull = rows * 32 / B;  // logical blocks of full rows only
-  row_ring<false, kRedStages>(&tin, nullptr, (rows + 31) / 32, 32, limit, status, [&](int64_t c, uint4* buf) {
+  row_ring<false, kRedStages>(&tin, nullptr, rows, (rows + 31) / 32, 32, limit, status, [&](int64_t c, uint4* buf) {
     V v[32];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {

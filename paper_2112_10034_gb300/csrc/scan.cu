@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(kRingWarps * 32, 2)
                      unsigned* status) {
   const int lane = threadIdx.x & 31;
   const int64_t rows = n / 32;
-  row_ring<true, rows_stages<R>()>(&tin, &tout, (rows + 31) / 32, 32, limit, status, [&](int64_t, uint4* buf) {
+  row_ring<true, rows_stages<R>()>(&tin, &tout, rows, (rows + 31) / 32, 32, limit, status, [&](int64_t, uint4* buf) {
     uint32_t w[32];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {  // unit j of row `lane` sits at unit j ^ (lane & 7)

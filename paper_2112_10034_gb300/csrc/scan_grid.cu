@@ -797,7 +797,8 @@ __global__ void __launch_bounds__(256) k_scan_grid_rows(const __grid_constant__ 
   if (tid == 0 && nbox > 0) tma_store_wait_read();  // the boxes have left shared memory
 }
 
-// BLOCK scope: the CTA is the logical block (persistent over blocks).
+// BLOCK scope, small or unaligned arrays: the CTA is the logical block
+// (persistent over blocks).
 template <class R>
 __global__ void __launch_bounds__(1024) k_scan_block(const uint32_t* __restrict__ in, uint32_t* __restrict__ out,
                                                      int64_t n, int excl) {
@@ -844,6 +845,144 @@ __global__ void __launch_bounds__(1024) k_scan_block(const uint32_t* __restrict_
   }
 }
 
+// BLOCK scope over aligned arrays: one row of 32 elements per lane, chunks of
+// `rpc` rows (whole logical blocks of rb = B / 32 rows, at most 32 rows) per
+// warp through row_ring.  A lane scans its row in registers (scan_row's
+// combines: the warp scan of k_scan_block), the block's rows are its rb
+// neighbouring lanes, whose totals are scanned by shuffles in the same
+// Hillis-Steele order, and every element takes prefix op value: the same
+// combines as k_scan_block, hence the same bits, without its three barriers
+// per block.  The partial last row (n % 32 elements) is read and written by
+// its lane from global memory.
+//
+// k_scan_block is bound by those barriers (4 bytes per thread between them);
+// this kernel by memory, and by issue for compensated sums.  2^26 fp32, B =
+// 32 / 256 / 1024: plain 334 / 197 / 225 -> 80 us (6700 GB/s), compensated
+// 430 / 280 / 289 -> 97 / 100 / 103 us.  Blocks that leave lanes idle (rpc <
+// 32) lose that share: B = 544 (17 rows) 259 -> 95 us plain.  Two chunks per
+// warp on three buffers; one chunk on one buffer measured 84 us at B = 256
+// plain and 113 us compensated.
+constexpr int kBlockScanStages = 3, kBlockScanChunks = 2;
+// Smaller arrays are bound by one row's latency, where k_scan_block's warp
+// scan ends sooner: 2^18 elements compensated 4.1 us against 6.2, 2^20 8.2
+// against 6.2; plain 10^3 3.2 against 4.0, 10^5 5.1 (B = 32) against 4.1.
+template <class R>
+constexpr int64_t block_rows_min() {
+  return R::kComp ? int64_t(1) << 19 : int64_t(1) << 16;
+}
+
+template <class R, bool EXCL>
+__global__ void __launch_bounds__(kRingWarps * 32, 2)
+    k_scan_block_rows(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtensorMap tout,
+                      const uint32_t* __restrict__ in, uint32_t* __restrict__ out, int64_t n, int rb, int rpc,
+                      uint32_t limit, unsigned* status) {
+  using T = typename R::T;
+  using V = typename R::V;
+  const int lane = threadIdx.x & 31;
+  const int pos = lane % rb;  // this lane's row within its logical block
+  const int64_t rows = n / 32, all_rows = (n + 31) / 32;
+  row_ring<true, kBlockScanStages>(&tin, &tout, rows, (all_rows + rpc - 1) / rpc, rpc, limit, status,
+                                         [&](int64_t c, uint4* buf) {
+    const int64_t row = c * rpc + lane;
+    const bool partial = lane < rpc && row == rows && rows < all_rows;
+    uint32_t w[32];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {  // unit j of row `lane` sits at unit j ^ (lane & 7)
+      const uint4 q = buf[lane * 8 + (j ^ (lane & 7))];
+      w[4 * j] = q.x;
+      w[4 * j + 1] = q.y;
+      w[4 * j + 2] = q.z;
+      w[4 * j + 3] = q.w;
+    }
+    if (partial) {
+#pragma unroll
+      for (int i = 0; i < 32; ++i) w[i] = row * 32 + i < n ? in[row * 32 + i] : to_bits(R::pad());
+    }
+    // the row's inclusive scan, its total, and the scan of the block's totals
+    uint64_t s[16], e[16];  // compensated: packed pairs
+    V v[32];                // otherwise
+    V tot;
+    if constexpr (R::kComp) {
+      float x[32];
+#pragma unroll
+      for (int i = 0; i < 32; ++i) x[i] = __uint_as_float(w[i]);
+      scan_row_pairs<32>(x, s, e);
+      float lo;
+      f2_unpack(s[15], lo, tot.s);
+      f2_unpack(e[15], lo, tot.e);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 32; ++i) v[i] = R::load(from_bits<T>(w[i]));
+      scan_row_regs<R, 32>(v);
+      tot = v[31];
+    }
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      if (d >= rb) break;
+      const V u = R::shfl_up(tot, d, 32);
+      if (pos >= d) tot = R::op(u, tot);
+    }
+    const V ex = R::shfl_up(tot, 1, 32);
+    const V pre = pos == 0 ? R::ident() : ex;
+    // every element: prefix op value (exclusive: the element before)
+    if constexpr (R::kComp) {
+      const uint64_t ps = f2_pack(pre.s, pre.s), pe = f2_pack(pre.e, pre.e);
+      float y[32];
+#pragma unroll
+      for (int k = 0; k < 16; ++k) {
+        uint64_t ns, t;
+        f2_two_sum(ps, s[k], ns, t);
+        f2_unpack(f2_add(ns, f2_add(f2_add(pe, e[k]), t)), y[2 * k], y[2 * k + 1]);
+      }
+      if constexpr (EXCL) {
+        w[0] = to_bits(R::out(pre));
+#pragma unroll
+        for (int i = 1; i < 32; ++i) w[i] = __float_as_uint(y[i - 1]);
+      } else {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) w[i] = __float_as_uint(y[i]);
+      }
+    } else {
+      if constexpr (EXCL) {
+        w[0] = to_bits(R::out(pre));
+#pragma unroll
+        for (int i = 1; i < 32; ++i) w[i] = to_bits(R::out(R::op(pre, v[i - 1])));
+      } else {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) w[i] = to_bits(R::out(R::op(pre, v[i])));
+      }
+    }
+    if (partial) {
+#pragma unroll
+      for (int i = 0; i < 32; ++i)
+        if (row * 32 + i < n) out[row * 32 + i] = w[i];
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      buf[lane * 8 + (j ^ (lane & 7))] = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
+  });
+}
+
+template <class R, bool EXCL>
+static cox_status launch_block_rows(const uint32_t* in, uint32_t* out, int64_t n, int block, cudaStream_t st) {
+  const int rb = block / 32, rpc = 32 / rb * rb;
+  CUtensorMap tin, tout;
+  if (!encode_rows32_map(&tin, in, n / 32, rpc) || !encode_rows32_map(&tout, out, n / 32, rpc)) return COX_ECUDA;
+  auto k = k_scan_block_rows<R, EXCL>;
+  constexpr size_t smem = ring_smem(kBlockScanStages);
+  static bool ready[kMaxDevices];  // per device: the kernel may take its shared memory
+  bool& rd = ready[device_index()];
+  if (!rd) {
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+      return COX_ECUDA;
+    rd = true;
+  }
+  const int64_t nch = ((n + 31) / 32 + rpc - 1) / rpc;
+  k<<<ring_grid(nch, kBlockScanChunks), kRingWarps * 32, smem, st>>>(tin, tout, in, out, n, rb, rpc,
+                                                                          spin_limit(), device_status_word());
+  return launch_status();
+}
+
 struct ScanWs {
   unsigned* ticket;
   uint32_t* flags;
@@ -873,6 +1012,8 @@ static cox_status launch_scan_scope(cox_scope scope, int block, const void* d_in
   const uint32_t* in = static_cast<const uint32_t*>(d_in);
   uint32_t* out = static_cast<uint32_t*>(d_out);
   if (scope == COX_SCOPE_BLOCK) {
+    if (n >= block_rows_min<R>() && n / 32 < (int64_t(1) << 31) && aligned16(d_in) && aligned16(d_out))
+      return excl ? launch_block_rows<R, true>(in, out, n, block, st) : launch_block_rows<R, false>(in, out, n, block, st);
     auto k = k_scan_block<R>;
     static int gmax[33];
     int& g = gmax[block / 32];
