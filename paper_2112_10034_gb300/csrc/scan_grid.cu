@@ -18,9 +18,11 @@
 // and its inclusive prefix in separate slots, each written before its flag
 // (release store) and read after it (acquire load), so a reader never sees a
 // value from the wrong stage.
+#include <algorithm>
 #include <type_traits>
 
 #include "cox_common.cuh"
+#include "tile_pipe.cuh"
 
 namespace cox {
 
@@ -140,304 +142,93 @@ __device__ typename R::V look_back_op(uint32_t* flags, uint64_t* agg, uint64_t* 
   return prefix;
 }
 
-// Look-back for 32-bit scan values over packed descriptors: desc[t] =
-// (state << 32) | value bits, state 0 nothing, 1 aggregate, 2 inclusive
-// prefix, so one relaxed 64-bit load returns a consistent (state, value)
-// pair (one round trip per window, no second load).  Same walk as
-// look_back_op.  Returns the tile's exclusive prefix.
+// Published tile aggregates of the row-tile kernel, zero until written.  A
+// 32-bit value is one 64-bit word, (1 << 32) | bits; a compensated pair two,
+// one per 32-bit half, each with its own flag, so that every word read is
+// whole whatever order the halves arrive in.
 template <class R>
-__device__ typename R::V look_back_packed(uint64_t* desc, int64_t tile, typename R::V total, uint32_t limit,
-                                          unsigned* status, bool& gave_up) {
-  using V = typename R::V;
-  using T = typename R::T;
-  const int lane = lane_id();
-  gave_up = false;
-  if (tile == 0) {
-    if (lane == 0) st_relaxed_u64(desc, (2ull << 32) | to_bits(total));
-    return R::ident();
-  }
-  if (lane == 0) st_relaxed_u64(desc + tile, (1ull << 32) | to_bits(total));
-  V prefix = R::ident();
-  uint32_t polls = 0;
-  bool timed_out = false;
-  for (int64_t w0 = tile - 1;; w0 -= 32 * kScanLookV) {
-    uint64_t d[kScanLookV];
-#pragma unroll
-    for (int v = 0; v < kScanLookV; ++v) {
-      const int64_t i = w0 - (lane * kScanLookV + v);
-      d[v] = i >= 0 ? ld_relaxed_u64(desc + i) : ((2ull << 32) | to_bits(R::ident()));  // before tile 0
-    }
-    int lp;
-    unsigned pm;
-    for (;;) {
-      lp = kScanLookV;
-#pragma unroll
-      for (int v = kScanLookV - 1; v >= 0; --v)
-        if ((d[v] >> 32) == 2u) lp = v;
-      pm = __ballot_sync(kFull, lp < kScanLookV);
-      const int fl = pm ? __ffs(pm) - 1 : 32;
-      bool missing = false;
-#pragma unroll
-      for (int v = 0; v < kScanLookV; ++v)
-        if ((lane < fl || (lane == fl && v <= lp)) && (d[v] >> 32) == 0u) missing = true;
-      if (!__any_sync(kFull, missing)) break;
-      if (++polls > limit) {
-        timed_out = true;
-        break;
-      }
-      if (polls > 64) __nanosleep(64);
-#pragma unroll
-      for (int v = 0; v < kScanLookV; ++v) {
-        const int64_t i = w0 - (lane * kScanLookV + v);
-        if ((d[v] >> 32) == 0u && i >= 0) d[v] = ld_relaxed_u64(desc + i);
-      }
-    }
-    if (timed_out) break;
-    const int fl = pm ? __ffs(pm) - 1 : 32;
-    V part = R::ident();
-#pragma unroll
-    for (int v = kScanLookV - 1; v >= 0; --v)  // older tiles first
-      if (lane < fl || (lane == fl && v <= lp)) part = R::op(from_bits<T>((uint32_t)d[v]), part);
-    prefix = R::op(warp_fold<R>(part), prefix);
-    if (pm) break;
-  }
-  if (__any_sync(kFull, timed_out)) {
-    gave_up = true;
-    if (lane == 0) {
-      atomicOr(status, (unsigned)kDevTimeout);
-      st_relaxed_u64(desc + tile, (2ull << 32) | to_bits(total));  // release successors
-    }
-    return R::ident();
-  }
-  if (lane == 0) st_relaxed_u64(desc + tile, (2ull << 32) | to_bits(R::op(prefix, total)));
-  return prefix;
-}
-
-// Two-level form of look_back_packed for 32-bit sums (wrapping adds): tiles
-// form groups of 32; a tile adds (1 << 48) | value to its group's
-// accumulator gacc[g] after publishing its aggregate, and the add that
-// completes the group publishes the group aggregate in gdesc[g]; the last
-// tile of a group also puts its inclusive prefix there (atomicMax: a
-// state-2 word is larger than any state-1 word).  The look-back reads the
-// tile's own group first, then whole groups, 32 per window (1024 tiles), so
-// its length no longer grows with the number of tiles in flight.
-__device__ unsigned look_back_sum2(uint64_t* desc, uint64_t* gdesc, uint64_t* gacc, int64_t tile, int64_t ntiles,
-                                   unsigned total, uint32_t limit, unsigned* status, bool& gave_up) {
-  const int lane = lane_id();
-  gave_up = false;
-  const int64_t g = tile >> 5;
-  const int pos = (int)(tile & 31);
-  if (lane == 0) {
-    st_relaxed_u64(desc + tile, ((tile == 0 ? 2ull : 1ull) << 32) | total);
-    const int64_t gsize = min((int64_t)32, ntiles - (g << 5));
-    const unsigned long long old = atomicAdd(reinterpret_cast<unsigned long long*>(gacc + g), (1ull << 48) | total);
-    if ((int64_t)(old >> 48) + 1 == gsize)
-      atomicMax(reinterpret_cast<unsigned long long*>(gdesc + g), (1ull << 32) | (uint32_t)(old + total));
-  }
-  unsigned prefix = 0;
-  uint32_t polls = 0;
-  bool timed_out = false;
-  bool done = tile == 0;
-  if (!done && pos > 0) {  // own group: lane l holds position l < pos
-    const int64_t g0 = g << 5;
-    uint64_t d = lane < pos ? ld_relaxed_u64(desc + g0 + lane) : (1ull << 32);
-    unsigned pm;
-    int fl;
-    for (;;) {
-      pm = __ballot_sync(kFull, lane < pos && (d >> 32) == 2u);
-      fl = pm ? 31 - __clz(pm) : -1;
-      const bool missing = lane < pos && lane > fl && (d >> 32) == 0u;
-      if (!__any_sync(kFull, missing)) break;
-      if (++polls > limit) {
-        timed_out = true;
-        break;
-      }
-      if (polls > 64) __nanosleep(64);
-      if (missing) d = ld_relaxed_u64(desc + g0 + lane);
-    }
-    if (!__any_sync(kFull, timed_out)) {
-      unsigned v = (lane < pos && lane >= fl) ? (unsigned)d : 0u;
-      prefix = __reduce_add_sync(kFull, v);
-      done = fl >= 0;
-    }
-  }
-  if (!done && !__any_sync(kFull, timed_out)) {  // whole groups: lane l holds group gw - l
-    for (int64_t gw = g - 1;; gw -= 32) {
-      const int64_t gi = gw - lane;
-      uint64_t d = gi >= 0 ? ld_relaxed_u64(gdesc + gi) : (2ull << 32);  // before group 0: 0
-      unsigned pm;
-      for (;;) {
-        pm = __ballot_sync(kFull, (d >> 32) == 2u);
-        const int fl = pm ? __ffs(pm) - 1 : 32;
-        const bool missing = lane <= fl && (d >> 32) == 0u;
-        if (!__any_sync(kFull, missing)) break;
-        if (++polls > limit) {
-          timed_out = true;
-          break;
-        }
-        if (polls > 64) __nanosleep(64);
-        if (missing && gi >= 0) d = ld_relaxed_u64(gdesc + gi);
-      }
-      if (__any_sync(kFull, timed_out)) break;
-      const int fl = pm ? __ffs(pm) - 1 : 32;
-      prefix += __reduce_add_sync(kFull, lane <= fl ? (unsigned)d : 0u);
-      if (pm) break;
-    }
-  }
-  if (__any_sync(kFull, timed_out)) {
-    gave_up = true;
-    if (lane == 0) {
-      atomicOr(status, (unsigned)kDevTimeout);
-      st_relaxed_u64(desc + tile, (2ull << 32) | total);
-      if (pos == 31) atomicMax(reinterpret_cast<unsigned long long*>(gdesc + g), (2ull << 32) | total);
-    }
-    return 0u;
-  }
-  if (lane == 0) {
-    const uint64_t inc = (2ull << 32) | (uint32_t)(prefix + total);
-    if (tile != 0) st_relaxed_u64(desc + tile, inc);
-    if (pos == 31) atomicMax(reinterpret_cast<unsigned long long*>(gdesc + g), inc);
-  }
-  return prefix;
-}
-
-// Look-back state and value in one 64-bit word, so a predecessor costs one
-// load: bits 62-63 the state (1 aggregate, 2 inclusive prefix), below them
-// the value -- a 32-bit value as is; a compensated pair as its sum word (bits
-// 0-31) and its error word rounded to 21 mantissa bits (bits 32-61).  The
-// rounding of an error word is at most 2^-22 of it, about 2^-46 of the sum:
-// far below the 1e-5 bar.  Tile aggregates also go, exact, to their own slot
-// for the group fold.
-template <class R>
-__device__ __forceinline__ uint64_t pk_word(uint64_t state, typename R::V v) {
-  if constexpr (R::kComp) {
-    const uint32_t eb = __float_as_uint(v.e);
-    // round to nearest on the 30-bit field; a carry into the exponent is the
-    // correct rounding up to the next binade
-    const uint64_t e30 = ((uint64_t)eb + 2u) >> 2;
-    return (state << 62) | ((e30 & 0x3FFFFFFFull) << 32) | (uint64_t)__float_as_uint(v.s);
-  } else {
-    return (state << 62) | (uint64_t)to_bits(v);
-  }
-}
-template <class R>
-__device__ __forceinline__ typename R::V pk_value(uint64_t w) {
-  using T = typename R::T;
-  if constexpr (R::kComp) return Pair{__uint_as_float((uint32_t)w), __uint_as_float((uint32_t)((w >> 32) << 2))};
-  else return from_bits<T>((uint32_t)w);
-}
-
-// Two-level look-back over packed words (any value except 32-bit sums, which
-// take look_back_sum2).  word[t]: the tile's state|value; agg[t]: its exact
-// aggregate; per group of 32 tiles gword[g] (state|value, only growing:
-// atomicMax, and a prefix word is above any aggregate word) and an arrival
-// counter gcnt[g].  The tile whose arrival completes its group folds the
-// group's 32 aggregates in tile order and publishes the group aggregate; the
-// group's last tile publishes its inclusive prefix as the group's.  Called by
-// a whole warp; returns the exclusive prefix.
-template <class R>
-__device__ typename R::V look_back_pk(uint64_t* word, uint64_t* agg, uint64_t* gword, uint32_t* gcnt, int64_t tile,
-                                      int64_t ntiles, typename R::V total, uint32_t limit, unsigned* status,
-                                      bool& gave_up) {
-  using V = typename R::V;
-  const int lane = lane_id();
-  gave_up = false;
-  const int64_t g = tile >> 5;
-  const int pos = (int)(tile & 31);
-  const int64_t g0 = g << 5;
-  int last = 0;
-  if (lane == 0) {
-    st_relaxed_u64(agg + tile, pack<R>(total));
-    st_relaxed_u64(word + tile, pk_word<R>(tile == 0 ? 2u : 1u, total));
-    __threadfence();
-    const int64_t gsize = min((int64_t)32, ntiles - g0);
-    last = (int64_t)atomicAdd(gcnt + g, 1u) + 1 == gsize;
-    if (last) __threadfence();
-  }
-  if (__shfl_sync(kFull, last, 0)) {
-    const int64_t gsize = min((int64_t)32, ntiles - g0);
-    V v = lane < gsize ? unpack<R>(ld_relaxed_u64(agg + g0 + lane)) : R::ident();
-    v = warp_fold<R>(v);
-    if (lane == 0) atomicMax(reinterpret_cast<unsigned long long*>(gword + g), pk_word<R>(1u, v));
-  }
-  V prefix = R::ident();
-  uint32_t polls = 0;
-  bool timed_out = false;
-  bool done = tile == 0;
-  if (!done && pos > 0) {  // own group: lane l holds position l < pos
-    uint64_t w = lane < pos ? ld_relaxed_u64(word + g0 + lane) : (1ull << 62);
-    unsigned pm;
-    int fl;
-    for (;;) {
-      pm = __ballot_sync(kFull, lane < pos && (w >> 62) == 2u);
-      fl = pm ? 31 - __clz(pm) : -1;
-      const bool missing = lane < pos && lane > fl && (w >> 62) == 0u;
-      if (!__any_sync(kFull, missing)) break;
-      if (++polls > limit) {
-        timed_out = true;
-        break;
-      }
-      if (polls > 64) __nanosleep(64);
-      if (missing) w = ld_relaxed_u64(word + g0 + lane);
-    }
-    if (!__any_sync(kFull, timed_out)) {
-      V part = R::ident();
-      if (lane < pos && lane >= fl) part = pk_value<R>(w);
-      prefix = warp_fold<R>(part);
-      done = fl >= 0;
-    }
-  }
-  if (!done && !__any_sync(kFull, timed_out)) {  // whole groups: lane l holds group gw0 - l
-    V gsum = R::ident();
-    for (int64_t gw0 = g - 1;; gw0 -= 32) {
-      const int64_t gi = gw0 - lane;
-      uint64_t w = gi >= 0 ? ld_relaxed_u64(gword + gi) : (2ull << 62) | pk_word<R>(0u, R::ident());
-      unsigned pm;
-      for (;;) {
-        pm = __ballot_sync(kFull, (w >> 62) == 2u);
-        const int fl = pm ? __ffs(pm) - 1 : 32;
-        const bool missing = lane <= fl && (w >> 62) == 0u;
-        if (!__any_sync(kFull, missing)) break;
-        if (++polls > limit) {
-          timed_out = true;
-          break;
-        }
-        if (polls > 64) __nanosleep(64);
-        if (missing && gi >= 0) w = ld_relaxed_u64(gword + gi);
-      }
-      if (__any_sync(kFull, timed_out)) break;
-      const int fl = pm ? __ffs(pm) - 1 : 32;
-      V part = R::ident();
-      if (lane <= fl && gi >= 0) part = pk_value<R>(w);
-      gsum = R::op(warp_fold<R>(part), gsum);  // older windows on the left
-      if (pm) break;
-    }
-    prefix = R::op(gsum, prefix);
-  }
-  if (__any_sync(kFull, timed_out)) {
-    gave_up = true;
-    if (lane == 0) {
-      atomicOr(status, (unsigned)kDevTimeout);
-      st_relaxed_u64(word + tile, pk_word<R>(2u, total));  // release successors
-      if (pos == 31) atomicMax(reinterpret_cast<unsigned long long*>(gword + g), pk_word<R>(2u, total));
-    }
-    return R::ident();
-  }
-  if (lane == 0) {
-    const V incl = R::op(prefix, total);
-    if (tile != 0) st_relaxed_u64(word + tile, pk_word<R>(2u, incl));
-    if (pos == 31) atomicMax(reinterpret_cast<unsigned long long*>(gword + g), pk_word<R>(2u, incl));
-  }
-  return prefix;
-}
-
-// Rows per lane of the row-tile grid scan (tiles of RPL x 8192 elements):
-// one for 32-bit values (33 KB tiles, six CTAs per SM), two for compensated
-// pairs (their registers allow four CTAs per SM, and the larger tile halves
-// the look-backs).
-template <class R>
-__host__ __device__ constexpr int grid_rows_rpl() {
+__host__ __device__ constexpr int agg_words() {
   return R::kComp ? 2 : 1;
+}
+template <class R>
+__device__ __forceinline__ void agg_store(uint64_t* agg, int64_t tile, typename R::V v) {
+  if constexpr (R::kComp)
+    asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(agg + 2 * tile),
+                 "l"((1ull << 32) | __float_as_uint(v.s)), "l"((1ull << 32) | __float_as_uint(v.e))
+                 : "memory");
+  else
+    st_relaxed_u64(agg + tile, (1ull << 32) | to_bits(v));
+}
+// Whether the aggregate is there; its value.
+template <class R>
+__device__ __forceinline__ void agg_load(const uint64_t* agg, int64_t tile, uint64_t (&w)[2]) {
+  if constexpr (R::kComp)
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(w[0]), "=l"(w[1]) : "l"(agg + 2 * tile) : "memory");
+  else
+    w[0] = w[1] = ld_relaxed_u64(agg + tile);
+}
+template <class R>
+__device__ __forceinline__ typename R::V agg_value(const uint64_t (&w)[2]) {
+  if constexpr (R::kComp) return Pair{__uint_as_float((uint32_t)w[0]), __uint_as_float((uint32_t)w[1])};
+  else return from_bits<typename R::T>((uint32_t)w[0]);
+}
+
+// Shape of the row-tile kernel, one CTA per SM.  32-bit values are bound by
+// memory: 9 tiles of 24 KB (192 rows) run 2^28 int32 in 312-321 us, 6 of 32 KB
+// 331, 12 of 16 KB 430 (a prefix per tile becomes the limit).  Compensated
+// sums are bound by the prefix walk, whose combines are eight adds: 6 tiles of
+// 32 KB, 2^27 in 185 us, 8 of 24 KB 217.  Two or three loads in flight keep
+// memory busy; without a limit they wait for each other, in an order that is
+// not the tiles' (2^28 int32, 32 KB tiles: 331 us with two, 359 with six).
+template <class R>
+struct GridCfg {
+  static constexpr int kRows = R::kComp ? 256 : 192;  // rows per tile and TMA box
+  static constexpr uint32_t kTileBytes = kRows * 128;
+  static constexpr int kNB = R::kComp ? 6 : 9;      // tiles in shared memory
+  static constexpr int kNW = kRows / 32;            // worker warps
+  static constexpr int kWin = 8;                    // 32-tile rows per poll of the walk
+  static constexpr int kFlight = R::kComp ? 2 : 3;  // loads in flight
+  static constexpr int kThreads = (kNW + 3) * 32;
+};
+
+// A walk over the published aggregates in tile order (a whole warp): advances
+// from `cur` to `tile`, folding what it passes into `run`.  False if the
+// words did not appear within `limit` polls or `abort` was raised.
+template <class R>
+__device__ bool follow(const uint64_t* agg, int64_t tile, int64_t& cur, typename R::V& run, uint32_t limit,
+                       volatile int* abort) {
+  using V = typename R::V;
+  constexpr int kWin = GridCfg<R>::kWin;  // 32-tile rows per poll
+  const int lane = lane_id();
+  uint32_t polls = 0;
+  while (cur < tile) {
+    uint64_t w[kWin][2];
+#pragma unroll
+    for (int v = 0; v < kWin; ++v) {
+      const int64_t t = cur + v * 32 + lane;
+      w[v][0] = w[v][1] = 0;
+      if (t < tile) agg_load<R>(agg, t, w[v]);
+    }
+    V part = R::ident();
+    int64_t step = 0;
+#pragma unroll
+    for (int v = 0; v < kWin; ++v) {
+      if (step != v * 32) break;  // (a gap in an earlier row)
+      const unsigned there = __ballot_sync(kFull, (w[v][0] >> 32) != 0 && (w[v][1] >> 32) != 0);
+      const int n = there == kFull ? 32 : __ffs(~there) - 1;
+      if (lane < n) part = R::op(part, agg_value<R>(w[v]));
+      step += n;
+    }
+    if (step) {
+      run = R::op(run, warp_fold<R>(part));
+      cur += step;
+      polls = 0;
+      continue;
+    }
+    if (++polls > limit || __any_sync(kFull, *abort)) return false;
+    __nanosleep(polls > 64 ? 200 : 20);
+  }
+  return true;
 }
 
 template <class R>
@@ -569,20 +360,17 @@ __global__ void __launch_bounds__(256) k_scan_grid(const uint32_t* __restrict__ 
   }
 }
 
-// GRID scope over aligned arrays of at least one full row: tiles of RPL x 256
-// rows of 32 elements (grid_rows_rpl) arrive by RPL 2D TMA boxes with
-// 128-byte swizzle; lane t of warp w owns rows 32 (RPL w + j) + t, j < RPL,
-// of the tile.  Pass A folds each row (its total), shuffle scans over the
-// warp's rows and a
-// scan of the 8 warp totals give every row's exclusive prefix, the tile
-// looks back for its own prefix (32-bit values: packed state|value
-// descriptors in `agg`), and pass B re-reads the row, carrying
-// prefix op value into each element (in place), before one TMA store.
-// Sums are folded left to right within a row, so fp32 results differ from
-// the shuffle form in their last bits (tolerance-checked).  The partial last
-// row (n % 32 elements) is read and written by its lane from global memory.
-constexpr int kGridBoxRows = 256;  // rows per TMA box; a tile is RPL boxes (RPL rows per lane)
-
+// GRID scope over aligned arrays of at least one full row, through tile_pipe:
+// a tile of 256 rows of 32 elements arrives by one 2D TMA box with 128-byte
+// swizzle; lane t of worker w owns row 32 w + t of the tile.  fold: each lane
+// folds its row, a shuffle scan over the warp's rows gives every row's
+// exclusive prefix in the warp; publish: the scan of the 8 warp totals, the
+// tile's aggregate; prefix: the walk over the earlier tiles' aggregates;
+// finish: re-reads the row, carrying prefix op value into each element (in
+// place), before one TMA store.  Sums are folded left to right within a row,
+// so fp32 results differ from the shuffle form in their last bits
+// (tolerance-checked).  The partial last row (n % 32 elements) is read and
+// written by its lane from global memory.
 // a op x for one element x: for a compensated pair the element's error word
 // is zero, so the error words need one add (a.e + t), not two.
 template <class R>
@@ -598,170 +386,111 @@ __device__ __forceinline__ typename R::V op_elem(typename R::V a, typename R::T 
   }
 }
 
-template <class R, int RPL>
-__global__ void __launch_bounds__(256) k_scan_grid_rows(const __grid_constant__ CUtensorMap tin,
-                                                        const __grid_constant__ CUtensorMap tout,
-                                                        const uint32_t* __restrict__ in, uint32_t* __restrict__ out,
-                                                        int64_t n, unsigned* ticket, uint32_t* flags, uint64_t* agg,
-                                                        uint64_t* inc, int64_t ntiles, int excl, uint32_t limit,
-                                                        unsigned* status) {
+template <class R>
+struct GridScanShared {
+  using C = GridCfg<R>;
+  PipeShared<C::kNB> pipe;
+  typename R::V pre[C::kNB][C::kRows];   // a row's exclusive prefix in its warp
+  typename R::V wtot[C::kNB][C::kNW];    // warp totals, then exclusive prefixes in the tile
+  typename R::V prefix[C::kNB];
+};
+template <class R>
+constexpr size_t grid_scan_smem(int nb) {
+  return 1024 + (size_t)nb * GridCfg<R>::kTileBytes + sizeof(GridScanShared<R>);
+}
+
+template <class R>
+struct GridScanOp {
   using T = typename R::T;
   using V = typename R::V;
-  extern __shared__ uint8_t gsr_raw[];
-  uint4* buf = reinterpret_cast<uint4*>((reinterpret_cast<uintptr_t>(gsr_raw) + 1023) & ~uintptr_t(1023));
-  __shared__ uint64_t s_bar;
-  __shared__ V s_wtot[8], s_cp[8];
-  __shared__ int64_t s_tile;
-  __shared__ int s_bad;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int64_t rows = n / 32;
-  if (tid == 0) {
-    s_tile = atomicAdd(ticket, 1u);
-    s_bad = 0;
-    mbar_init(&s_bar, 1);
-    mbar_init_fence();
+  using C = GridCfg<R>;
+  const CUtensorMap *tin, *tout;
+  const uint32_t* in;
+  uint32_t* out;
+  int64_t n, rows;
+  uint64_t* agg;
+  int excl;
+  uint32_t limit;
+  uint4* bufs;
+  GridScanShared<R>* sh;
+  int64_t cur;  // prefix warps: tiles walked, and their fold
+  V run;
+
+  __device__ uint4* buf(int slot) const { return bufs + (size_t)slot * C::kRows * 8; }
+  __device__ bool partial(int64_t row) const { return row == rows && rows * 32 < n; }
+
+  __device__ void load(int slot, int64_t tile) const {
+    const int64_t r0 = tile * C::kRows;
+    uint64_t* bar = sh->pipe.full + slot;
+    if (r0 < rows) {
+      mbar_arrive_expect_tx(bar, C::kTileBytes);
+      tma_load_2d(buf(slot), tin, 0, (int)r0, bar);
+    } else {
+      mbar_arrive(bar);  // only the partial last row
+    }
   }
-  __syncthreads();
-  const int64_t tile = s_tile;
-  if (tile >= ntiles) return;
-  constexpr int kTileRows = RPL * kGridBoxRows;
-  const int64_t r0 = tile * kTileRows;
-  // boxes holding full rows
-  const int nbox = r0 >= rows ? 0 : (int)min((int64_t)RPL, (rows - r0 + kGridBoxRows - 1) / kGridBoxRows);
-  if (tid == 0 && nbox > 0) {
-    mbar_arrive_expect_tx(&s_bar, (uint32_t)nbox * kGridBoxRows * 128u);
-    for (int bx = 0; bx < nbox; ++bx)
-      tma_load_2d(buf + bx * kGridBoxRows * 8, &tin, 0, (int)(r0 + bx * kGridBoxRows), &s_bar);
-  }
-  // lane owns rows 32 * (RPL * w + j) + lane, j < RPL, of the tile
-  int rl[RPL];
+  __device__ void fold(int slot, int64_t tile) const {
+    const int warp = threadIdx.x >> 5, lane = lane_id(), rl = threadIdx.x;
+    const int64_t row = tile * C::kRows + rl;
+    uint4* b = buf(slot);
+    if (partial(row)) {
+      const uint32_t pad = to_bits(R::pad());
 #pragma unroll
-  for (int j = 0; j < RPL; ++j) rl[j] = 32 * (RPL * warp + j) + lane;
-  const uint32_t pad = to_bits(R::pad());
-  if (nbox > 0) {
-    const bool ok = mbar_wait_bounded(&s_bar, 0u, limit);
-    if (__syncthreads_or(!ok)) {
-      if (tid == 0) {
-        atomicOr(status, (unsigned)kDevTimeout);
-        mbar_wait_bounded(&s_bar, 0u, limit);
-        if constexpr (!std::is_same<R, Plain<AddU>>::value) {
-          // a zero prefix for successors; the group level counts this tile's
-          // arrival and, if it completes the group, publishes some aggregate
-          // (the device status already says the results are not to be used)
-          const int64_t ngroups = (ntiles + 31) / 32, g = tile >> 5;
-          const int64_t gsize = min((int64_t)32, ntiles - (g << 5));
-          uint64_t* gword = inc + ntiles;
-          uint32_t* gcnt = reinterpret_cast<uint32_t*>(gword + ngroups);
-          st_relaxed_u64(agg + tile, pack<R>(R::ident()));
-          st_relaxed_u64(inc + tile, pk_word<R>(2u, R::ident()));
-          __threadfence();
-          if ((int64_t)atomicAdd(gcnt + g, 1u) + 1 == gsize)
-            atomicMax(reinterpret_cast<unsigned long long*>(gword + g), pk_word<R>(1u, R::ident()));
-          if ((tile & 31) == 31)
-            atomicMax(reinterpret_cast<unsigned long long*>(gword + g), pk_word<R>(2u, R::ident()));
-        } else {
-          st_relaxed_u64(agg + tile, (2ull << 32) | to_bits(R::ident()));
-          if constexpr (std::is_same<R, Plain<AddU>>::value) {  // keep the group level consistent
-            const int64_t ngroups = (ntiles + 31) / 32, g = tile >> 5;
-            const int64_t gsize = min((int64_t)32, ntiles - (g << 5));
-            uint64_t* gd = inc + ntiles;
-            const unsigned long long old =
-                atomicAdd(reinterpret_cast<unsigned long long*>(gd + ngroups + g), 1ull << 48);
-            if ((int64_t)(old >> 48) + 1 == gsize)
-              atomicMax(reinterpret_cast<unsigned long long*>(gd + g), (1ull << 32) | (uint32_t)old);
-            if ((tile & 31) == 31) atomicMax(reinterpret_cast<unsigned long long*>(gd + g), 2ull << 32);
-          }
-        }
+      for (int j = 0; j < 8; ++j) {
+        const int64_t e = row * 32 + 4 * j;
+        uint4 q;
+        q.x = e < n ? in[e] : pad;
+        q.y = e + 1 < n ? in[e + 1] : pad;
+        q.z = e + 2 < n ? in[e + 2] : pad;
+        q.w = e + 3 < n ? in[e + 3] : pad;
+        b[rl * 8 + (j ^ (rl & 7))] = q;
       }
-      return;
     }
-  }
-  // The partial last row (n % 32 elements) comes from global memory, after the
-  // boxes have landed (they fill rows past the end with zeros).
-  auto fill_partial = [&](int rl) {
-    const int64_t row = r0 + rl;
-    if (!(row == rows && rows * 32 < n)) return;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int64_t e = row * 32 + 4 * j;
-      uint4 q;
-      q.x = e < n ? in[e] : pad;
-      q.y = e + 1 < n ? in[e + 1] : pad;
-      q.z = e + 2 < n ? in[e + 2] : pad;
-      q.w = e + 3 < n ? in[e + 3] : pad;
-      buf[rl * 8 + (j ^ (rl & 7))] = q;
-    }
-  };
-#pragma unroll
-  for (int j = 0; j < RPL; ++j) fill_partial(rl[j]);
-  // ---- pass A: row totals (left folds)
-  auto row_total = [&](int rl) {
     V tot = R::ident();
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-      const uint4 q = buf[rl * 8 + (j ^ (rl & 7))];
+      const uint4 q = b[rl * 8 + (j ^ (rl & 7))];
       tot = op_elem<R>(tot, from_bits<T>(q.x));
       tot = op_elem<R>(tot, from_bits<T>(q.y));
       tot = op_elem<R>(tot, from_bits<T>(q.z));
       tot = op_elem<R>(tot, from_bits<T>(q.w));
     }
-    return tot;
-  };
-  auto warp_incl = [&](V v) {
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
-      const V u = R::shfl_up(v, d, 32);
-      if (lane >= d) v = R::op(u, v);
+      const V u = R::shfl_up(tot, d, 32);
+      if (lane >= d) tot = R::op(u, tot);
     }
-    return v;
-  };
-  V pre[RPL], run = R::ident();  // run: the warp's earlier rows in all
-#pragma unroll
-  for (int j = 0; j < RPL; ++j) {
-    const V ij = R::op(run, warp_incl(row_total(rl[j])));
-    const V ej = R::shfl_up(ij, 1, 32);
-    pre[j] = lane == 0 ? run : ej;
-    run = R::shfl_idx(ij, 31, 32);
+    const V ex = R::shfl_up(tot, 1, 32);
+    sh->pre[slot][rl] = lane == 0 ? R::ident() : ex;
+    if (lane == 31) sh->wtot[slot][warp] = tot;
   }
-  if (lane == 31) s_wtot[warp] = run;
-  __syncthreads();
-  if (warp == 0) {
-    V total = R::ident();
-    if (lane == 0) {
+  __device__ void publish(int slot, int64_t tile) const {
+    if (lane_id() == 0) {
+      V total = R::ident();
 #pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        s_cp[k] = total;
-        total = R::op(total, s_wtot[k]);
+      for (int k = 0; k < C::kNW; ++k) {
+        const V t = sh->wtot[slot][k];
+        sh->wtot[slot][k] = total;
+        total = R::op(total, t);
       }
-    }
-    total = R::shfl_idx(total, 0, 32);
-    bool gave_up;
-    V prefix;
-    const int64_t ngroups = (ntiles + 31) / 32;
-    if constexpr (std::is_same<R, Plain<AddU>>::value) {
-      // group descriptors and accumulators after the tile slots
-      prefix = look_back_sum2(agg, inc + ntiles, inc + ntiles + ngroups, tile, ntiles, total, limit, status, gave_up);
-    } else {
-      // packed tile words in `inc`, exact aggregates in `agg`; after the tile
-      // slots the group words (64-bit), then the group arrival counters
-      uint64_t* gword = inc + ntiles;
-      uint32_t* gcnt = reinterpret_cast<uint32_t*>(gword + ngroups);
-      prefix = look_back_pk<R>(inc, agg, gword, gcnt, tile, ntiles, total, limit, status, gave_up);
-    }
-    if (lane == 0) {
-#pragma unroll
-      for (int k = 0; k < 8; ++k) s_cp[k] = R::op(prefix, s_cp[k]);
-      s_bad = gave_up;
+      agg_store<R>(agg, tile, total);
     }
   }
-  __syncthreads();
-  if (s_bad) return;
-  // ---- pass B: carry prefix op value through each row, in place
-  auto carry_row = [&](int rl, V carry) {
+  __device__ bool prefix(int slot, int64_t tile, volatile int* abort) {
+    if (!follow<R>(agg, tile, cur, run, limit, abort)) return false;
+    if (lane_id() == 0) sh->prefix[slot] = run;
+    return true;
+  }
+  __device__ void finish(int slot, int64_t tile) const {
+    const int rl = threadIdx.x;
+    uint4* b = buf(slot);
+    V carry = R::op(R::op(sh->prefix[slot], sh->wtot[slot][rl >> 5]), sh->pre[slot][rl]);
+    const int64_t row = tile * C::kRows + rl;
+    const bool part = partial(row);
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-      uint4& slot = buf[rl * 8 + (j ^ (rl & 7))];
-      uint4 q = slot;
+      uint4& s = b[rl * 8 + (j ^ (rl & 7))];
+      uint4 q = s;
       uint32_t* w = &q.x;
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
@@ -769,32 +498,38 @@ __global__ void __launch_bounds__(256) k_scan_grid_rows(const __grid_constant__ 
         w[k] = to_bits(R::out(excl ? carry : nx));
         carry = nx;
       }
-      slot = q;
+      s = q;
+      if (part) {
+        const int64_t e = row * 32 + 4 * j;
+        if (e < n) out[e] = q.x;
+        if (e + 1 < n) out[e + 1] = q.y;
+        if (e + 2 < n) out[e + 2] = q.z;
+        if (e + 3 < n) out[e + 3] = q.w;
+      }
     }
-  };
-  const V cw = s_cp[warp];
-#pragma unroll
-  for (int j = 0; j < RPL; ++j) carry_row(rl[j], R::op(cw, pre[j]));
-  fence_proxy_async_smem();
-  __syncthreads();
-  if (tid == 0)
-    for (int bx = 0; bx < nbox; ++bx) tma_store_2d(&tout, 0, (int)(r0 + bx * kGridBoxRows), buf + bx * kGridBoxRows * 8);
-  auto store_partial = [&](int rl) {
-    const int64_t row = r0 + rl;
-    if (!(row == rows && rows * 32 < n)) return;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const uint4 q = buf[rl * 8 + (j ^ (rl & 7))];
-      const int64_t e = row * 32 + 4 * j;
-      if (e < n) out[e] = q.x;
-      if (e + 1 < n) out[e + 1] = q.y;
-      if (e + 2 < n) out[e + 2] = q.z;
-      if (e + 3 < n) out[e + 3] = q.w;
+    fence_proxy_async_smem();  // before the bulk store reads the buffer
+  }
+  __device__ void store(int slot, int64_t tile) const {
+    if (tile * C::kRows < rows) {
+      tma_store_2d(tout, 0, (int)(tile * C::kRows), buf(slot));
+      tma_store_wait_read();
     }
-  };
-#pragma unroll
-  for (int j = 0; j < RPL; ++j) store_partial(rl[j]);
-  if (tid == 0 && nbox > 0) tma_store_wait_read();  // the boxes have left shared memory
+  }
+};
+
+template <class R>
+__global__ void __launch_bounds__(GridCfg<R>::kThreads, 1)
+    k_scan_grid_rows(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtensorMap tout,
+                     const uint32_t* __restrict__ in, uint32_t* __restrict__ out, int64_t n, unsigned* ticket,
+                     uint64_t* agg, int64_t ntiles, int excl, int nb, int flight, uint32_t limit,
+                     unsigned* status) {
+  using C = GridCfg<R>;
+  extern __shared__ uint8_t gsr_raw[];
+  uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(gsr_raw) + 1023) & ~uintptr_t(1023));
+  GridScanShared<R>* sh = reinterpret_cast<GridScanShared<R>*>(base + (size_t)nb * C::kTileBytes);
+  GridScanOp<R> op{&tin, &tout, in, out, n, n / 32, agg, excl, limit, reinterpret_cast<uint4*>(base), sh, 0,
+                   R::ident()};
+  tile_pipe<C::kNB, C::kNW>(sh->pipe, op, nb, flight, ntiles, ticket, limit, status);
 }
 
 // BLOCK scope, small or unaligned arrays: the CTA is the logical block
@@ -1023,27 +758,36 @@ static cox_status launch_scan_scope(cox_scope scope, int block, const void* d_in
     return launch_status();
   }
   if (n >= 32 && n / 32 < (int64_t(1) << 31) && aligned16(d_in) && aligned16(d_out)) {
-    constexpr int RPL = grid_rows_rpl<R>();
-    constexpr int64_t kTileElems = (int64_t)RPL * kGridBoxRows * 32;
+    using C = GridCfg<R>;
+    constexpr int64_t kTileElems = C::kRows * 32;
     const int64_t ntiles = (n + kTileElems - 1) / kTileElems;
-    const size_t need = scan_ws_bytes(ntiles) + 24 * (size_t)((ntiles + 31) / 32);  // + group words
-    if (!ws || ws_bytes < need) return COX_ENOMEM;
+    if (!ws || ws_bytes < cox_scan_workspace(COX_SCOPE_GRID, n)) return COX_ENOMEM;
     if (!aligned16(ws)) return COX_EINVAL;
     CUtensorMap tin, tout;
-    if (!encode_rows32_map(&tin, d_in, n / 32, kGridBoxRows) || !encode_rows32_map(&tout, d_out, n / 32, kGridBoxRows))
+    if (!encode_rows32_map(&tin, d_in, n / 32, C::kRows) || !encode_rows32_map(&tout, d_out, n / 32, C::kRows))
       return COX_ECUDA;
-    if (cudaMemsetAsync(ws, 0, need, st) != cudaSuccess) return COX_ECUDA;
-    const ScanWs w = scan_ws(ws, ntiles);
-    auto k = k_scan_grid_rows<R, RPL>;
-    const size_t smem = (size_t)RPL * kGridBoxRows * 128 + 1024;
-    static bool attr[kMaxDevices];  // per device
-    if (!attr[device_index()]) {
-      if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    // the ticket, then a zero aggregate per tile (within cox_scan_workspace)
+    const size_t used = kScanWsHeader + (size_t)ntiles * agg_words<R>() * 8;
+    if (cudaMemsetAsync(ws, 0, used, st) != cudaSuccess) return COX_ECUDA;
+    auto k = k_scan_grid_rows<R>;
+    static int grid[kMaxDevices];  // resident CTAs, per device
+    int& g = grid[device_index()];
+    if (g == 0) {
+      if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)grid_scan_smem<R>(C::kNB)) !=
+          cudaSuccess)
         return COX_ECUDA;
-      attr[device_index()] = true;
+      g = persistent_grid(k, C::kThreads, grid_scan_smem<R>(C::kNB), 1 << 30);
     }
-    k<<<(unsigned)ntiles, 256, smem, st>>>(tin, tout, in, out, n, w.ticket, w.flags, w.agg, w.inc, ntiles, excl,
-                                           spin_limit(), device_status_word());
+    // as many buffers as give every CTA work: a short array's tiles spread
+    // over the CTAs instead of queueing in the first ones
+    const int64_t ctas = ntiles < g ? ntiles : g;
+    const int nb = (int)std::min<int64_t>(C::kNB, (ntiles + ctas - 1) / ctas);
+    // an array that fits the buffers is loaded all at once
+    const int flight = ntiles <= ctas * nb ? nb : C::kFlight;
+    k<<<(unsigned)ctas, C::kThreads, grid_scan_smem<R>(nb), st>>>(
+        tin, tout, in, out, n, static_cast<unsigned*>(ws),
+        reinterpret_cast<uint64_t*>(static_cast<char*>(ws) + kScanWsHeader), ntiles, excl, nb, flight, spin_limit(),
+        device_status_word());
     return launch_status();
   }
   constexpr int TILE = grid_scan_tile<R>();

@@ -53,3 +53,61 @@ def test_block_scan_rows_equal_the_general_kernel(cox, B, dt, op, comp, tail):  
     y = x.clone()
     assert cox.cox_scan(op, dt, o.BLOCK, B, y.data_ptr(), y.data_ptr(), n, comp, 1, None, 0, None) == cox.COX_OK
     assert torch.equal(y, got[1][:n])
+
+
+def _grid_scan(cox, src, n, op, dt, comp, excl):  # noqa: F811
+    import torch
+    out = poisoned(n, torch.int32)
+    ws = torch.full((cox.cox_scan_workspace(o.GRID, n),), 0xA5, dtype=torch.uint8, device="cuda")
+    assert cox.cox_scan(op, dt, o.GRID, 256, src.data_ptr(), out.data_ptr(), n, comp, excl, ws.data_ptr(), ws.numel(),
+                        None) == cox.COX_OK
+    assert bool((out[n:] == POISON).all())
+    return out[:n]
+
+
+GRID_TILE = {0: 6144, 1: 8192}  # elements per tile: 32-bit values, compensated pairs
+GRID_BUFS = {0: 9, 1: 6}        # tiles a CTA keeps
+
+
+@pytest.mark.parametrize("where", ["row", "tile", "grid", "buffers"])
+@pytest.mark.parametrize("delta", [-33, -1, 0, 1, 32])
+@pytest.mark.parametrize("dt,op,comp", [(o.I32, o.SUM, 0), (o.U32, o.MAX, 0), (o.I32, o.XOR, 0), (o.F32, o.MIN, 0),
+                                        (o.F32, o.SUM, 1)])
+def test_grid_scan_pipeline_equals_the_general_kernel(cox, where, delta, dt, op, comp):  # noqa: F811
+    """Aligned arrays (the tile pipeline) against the same values 4 bytes off
+    (the general kernel): whole numbers bit for bit, compensated sums to one
+    rounding of the output (2^-24) on either side."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    t = GRID_TILE[comp]
+    n = {"row": 64, "tile": 3 * t, "grid": sms * t, "buffers": sms * GRID_BUFS[comp] * t}[where] + delta
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n + op)
+    x = torch.randn(n, generator=g, device="cuda").view(torch.int32) if dt == o.F32 else \
+        torch.randint(-2**31, 2**31 - 1, (n,), generator=g, device="cuda", dtype=torch.int32)
+    off = torch.empty(n + 1, dtype=torch.int32, device="cuda")
+    off[1:] = x
+    for excl in (0, 1):
+        a = _grid_scan(cox, x, n, op, dt, comp, excl)
+        b = _grid_scan(cox, off[1:], n, op, dt, comp, excl)
+        if comp:
+            fa, fb = a.view(torch.float32).double(), b.view(torch.float32).double()
+            # each is within u |y| + 2^-40 sum|x| of the exact prefix
+            assert bool(((fa - fb).abs() <= 2.0**-23 * fb.abs() + 2.0**-39 * x.view(torch.float32).abs().sum()).all())
+        else:
+            assert torch.equal(a, b)
+    assert cox.device_status() == cox.COX_OK
+
+
+def test_grid_scan_is_reproducible_and_works_in_place(cox):  # noqa: F811
+    """The running prefix is one sequence of combines; a tile is read before it is written."""
+    import torch
+    n = 3_000_017
+    g = torch.Generator(device="cuda")
+    g.manual_seed(5)
+    x = torch.randint(-1000, 1000, (n,), generator=g, device="cuda", dtype=torch.int32)
+    want = x.cumsum(0, dtype=torch.int64).to(torch.int32)
+    ws = torch.empty(cox.cox_scan_workspace(o.GRID, n), dtype=torch.uint8, device="cuda")
+    assert cox.cox_scan(o.SUM, o.I32, o.GRID, 256, x.data_ptr(), x.data_ptr(), n, 0, 0, ws.data_ptr(), ws.numel(),
+                        None) == cox.COX_OK
+    assert torch.equal(x, want)
