@@ -5,11 +5,11 @@
 // shared memory, warp 0 scans them, and every element takes its warp's
 // prefix (the uniform_add step).
 //
-// GRID scope chains tiles with a decoupled look-back.  16-byte aligned
-// arrays take the row-tile kernel (k_scan_grid_rows, below); in any other
-// layout a CTA takes a tile (16384 elements; 8192 for compensated sums,
-// whose pairs need twice the shared memory) from an atomic ticket, receives
-// it by one TMA bulk copy,
+// GRID scope chains tiles.  16-byte aligned arrays take the row-tile kernels
+// (k_scan_grid_rows and k_scan_grid_short, below); in any other layout tiles
+// are chained by a decoupled look-back: a CTA takes a tile (16384 elements;
+// 8192 for compensated sums, whose pairs need twice the shared memory) from an
+// atomic ticket, receives it by plain loads (or one TMA bulk copy),
 // and every warp scans its rows of 32 elements with shfl_up, carrying row
 // totals across its rows (eight rows at a time for instruction-level
 // parallelism).  Lane 0 of warp 0 scans the eight warp totals, the tile
@@ -386,33 +386,30 @@ __device__ __forceinline__ typename R::V op_elem(typename R::V a, typename R::T 
   }
 }
 
-template <class R>
+template <class R, class C>
 struct GridScanShared {
-  using C = GridCfg<R>;
   PipeShared<C::kNB> pipe;
-  typename R::V pre[C::kNB][C::kRows];   // a row's exclusive prefix in its warp
-  typename R::V wtot[C::kNB][C::kNW];    // warp totals, then exclusive prefixes in the tile
+  typename R::V pre[C::kNB][C::kRows];  // a row's exclusive prefix in its warp
+  typename R::V wtot[C::kNB][C::kNW];   // warp totals, then exclusive prefixes in the tile
   typename R::V prefix[C::kNB];
 };
-template <class R>
+template <class R, class C>
 constexpr size_t grid_scan_smem(int nb) {
-  return 1024 + (size_t)nb * GridCfg<R>::kTileBytes + sizeof(GridScanShared<R>);
+  return 1024 + (size_t)nb * C::kTileBytes + sizeof(GridScanShared<R, C>);
 }
 
-template <class R>
+template <class R, class C>
 struct GridScanOp {
   using T = typename R::T;
   using V = typename R::V;
-  using C = GridCfg<R>;
   const CUtensorMap *tin, *tout;
   const uint32_t* in;
   uint32_t* out;
   int64_t n, rows;
   uint64_t* agg;
   int excl;
-  uint32_t limit;
   uint4* bufs;
-  GridScanShared<R>* sh;
+  GridScanShared<R, C>* sh;
   int64_t cur;  // prefix warps: tiles walked, and their fold
   V run;
 
@@ -476,7 +473,7 @@ struct GridScanOp {
       agg_store<R>(agg, tile, total);
     }
   }
-  __device__ bool prefix(int slot, int64_t tile, volatile int* abort) {
+  __device__ bool prefix(int slot, int64_t tile, uint32_t limit, volatile int* abort) {
     if (!follow<R>(agg, tile, cur, run, limit, abort)) return false;
     if (lane_id() == 0) sh->prefix[slot] = run;
     return true;
@@ -526,10 +523,89 @@ __global__ void __launch_bounds__(GridCfg<R>::kThreads, 1)
   using C = GridCfg<R>;
   extern __shared__ uint8_t gsr_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(gsr_raw) + 1023) & ~uintptr_t(1023));
-  GridScanShared<R>* sh = reinterpret_cast<GridScanShared<R>*>(base + (size_t)nb * C::kTileBytes);
-  GridScanOp<R> op{&tin, &tout, in, out, n, n / 32, agg, excl, limit, reinterpret_cast<uint4*>(base), sh, 0,
+  GridScanShared<R, C>* sh = reinterpret_cast<GridScanShared<R, C>*>(base + (size_t)nb * C::kTileBytes);
+  GridScanOp<R, C> op{&tin, &tout, in, out, n, n / 32, agg, excl, reinterpret_cast<uint4*>(base), sh, 0,
                    R::ident()};
-  tile_pipe<C::kNB, C::kNW>(sh->pipe, op, nb, flight, ntiles, ticket, limit, status);
+  tile_pipe<C::kNB, C::kNW, 1>(sh->pipe, op, nb, flight, ntiles, ticket, limit, status);
+}
+
+// Short arrays, whose tiles are all resident at once: one tile per CTA in the
+// same three parts, several CTAs per SM, and the prefix gathered by all warps
+// together (every earlier aggregate read once, in one round trip when they
+// are there).  The pipeline serves an SM's tiles one after the other, which
+// costs about a microsecond each.
+struct GridShortCfg {
+  static constexpr int kRows = 256, kNB = 1, kNW = kRows / 32;
+  static constexpr uint32_t kTileBytes = kRows * 128;
+};
+
+template <class R>
+__global__ void __launch_bounds__(GridShortCfg::kNW * 32)
+    k_scan_grid_short(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtensorMap tout,
+                      const uint32_t* __restrict__ in, uint32_t* __restrict__ out, int64_t n, unsigned* ticket,
+                      uint64_t* agg, int excl, uint32_t limit, unsigned* status) {
+  using C = GridShortCfg;
+  using V = typename R::V;
+  extern __shared__ uint8_t gsr_raw[];
+  uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(gsr_raw) + 1023) & ~uintptr_t(1023));
+  GridScanShared<R, C>* sh = reinterpret_cast<GridScanShared<R, C>*>(base + C::kTileBytes);
+  __shared__ int64_t s_tile;
+  __shared__ V s_part[C::kNW];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  GridScanOp<R, C> op{&tin, &tout, in, out, n, n / 32, agg, excl, reinterpret_cast<uint4*>(base), sh, 0,
+                      R::ident()};
+  if (tid == 0) {
+    mbar_init(sh->pipe.full, 1);
+    mbar_init_fence();
+    const int64_t t = (int64_t)atomicAdd(ticket, 1u);
+    op.load(0, t);
+    s_tile = t;
+  }
+  __syncthreads();
+  const int64_t tile = s_tile;
+  if (__syncthreads_or(!mbar_wait_bounded(sh->pipe.full, 0u, limit))) {
+    if (tid == 0) {
+      atomicOr(status, (unsigned)kDevTimeout);
+      mbar_wait_bounded(sh->pipe.full, 0u, limit);
+    }
+    return;
+  }
+  op.fold(0, tile);
+  __syncthreads();
+  if (warp == 0) op.publish(0, tile);
+  V part = R::ident();
+  bool ok = true;
+  for (int64_t t = tid; t < tile; t += C::kNW * 32) {
+    uint64_t w[2];
+    for (uint32_t polls = 0;; ++polls) {
+      agg_load<R>(agg, t, w);
+      if ((w[0] >> 32) != 0 && (w[1] >> 32) != 0) break;
+      if (polls > limit) {
+        ok = false;
+        break;
+      }
+      __nanosleep(polls > 64 ? 200 : 20);
+    }
+    if (!ok) break;
+    part = R::op(part, agg_value<R>(w));
+  }
+  __syncwarp();
+  part = warp_fold<R>(part);
+  if (lane == 0) s_part[warp] = part;
+  if (__syncthreads_or(!ok)) {
+    if (tid == 0) atomicOr(status, (unsigned)kDevTimeout);
+    return;
+  }
+  if (tid == 0) {
+    V p = R::ident();
+#pragma unroll
+    for (int k = 0; k < C::kNW; ++k) p = R::op(p, s_part[k]);
+    sh->prefix[0] = p;
+  }
+  __syncthreads();
+  op.finish(0, tile);
+  __syncthreads();
+  if (tid == 0) op.store(0, tile);
 }
 
 // BLOCK scope, small or unaligned arrays: the CTA is the logical block
@@ -758,36 +834,47 @@ static cox_status launch_scan_scope(cox_scope scope, int block, const void* d_in
     return launch_status();
   }
   if (n >= 32 && n / 32 < (int64_t(1) << 31) && aligned16(d_in) && aligned16(d_out)) {
-    using C = GridCfg<R>;
-    constexpr int64_t kTileElems = C::kRows * 32;
-    const int64_t ntiles = (n + kTileElems - 1) / kTileElems;
     if (!ws || ws_bytes < cox_scan_workspace(COX_SCOPE_GRID, n)) return COX_ENOMEM;
     if (!aligned16(ws)) return COX_EINVAL;
+    // Little more than one resident wave of one-tile CTAs (six per SM), or the
+    // pipeline.  2^22 int32 16.9 us against 20.2, 2^23 25.6 against 29.0, 1.26 x
+    // 10^7 31.7 against 30.5, 2^24 37.7 against 35.9; the smallest arrays also
+    // start sooner (10^4: 7.4 against 8.6).
+    const int64_t short_tiles = (n + GridShortCfg::kRows * 32 - 1) / (GridShortCfg::kRows * 32);
+    const bool use_short = short_tiles <= (int64_t)8 * sm_count();
+    using C = GridCfg<R>;
+    const int rows = use_short ? GridShortCfg::kRows : C::kRows;
+    const int64_t ntiles = use_short ? short_tiles : (n + C::kRows * 32 - 1) / (C::kRows * 32);
     CUtensorMap tin, tout;
-    if (!encode_rows32_map(&tin, d_in, n / 32, C::kRows) || !encode_rows32_map(&tout, d_out, n / 32, C::kRows))
+    if (!encode_rows32_map(&tin, d_in, n / 32, rows) || !encode_rows32_map(&tout, d_out, n / 32, rows))
       return COX_ECUDA;
     // the ticket, then a zero aggregate per tile (within cox_scan_workspace)
-    const size_t used = kScanWsHeader + (size_t)ntiles * agg_words<R>() * 8;
-    if (cudaMemsetAsync(ws, 0, used, st) != cudaSuccess) return COX_ECUDA;
+    if (cudaMemsetAsync(ws, 0, kScanWsHeader + (size_t)ntiles * agg_words<R>() * 8, st) != cudaSuccess)
+      return COX_ECUDA;
+    unsigned* ticket = static_cast<unsigned*>(ws);
+    uint64_t* agg = reinterpret_cast<uint64_t*>(static_cast<char*>(ws) + kScanWsHeader);
+    if (use_short) {
+      k_scan_grid_short<R><<<(unsigned)ntiles, GridShortCfg::kNW * 32, grid_scan_smem<R, GridShortCfg>(1), st>>>(
+          tin, tout, in, out, n, ticket, agg, excl, spin_limit(), device_status_word());
+      return launch_status();
+    }
     auto k = k_scan_grid_rows<R>;
     static int grid[kMaxDevices];  // resident CTAs, per device
     int& g = grid[device_index()];
     if (g == 0) {
-      if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)grid_scan_smem<R>(C::kNB)) !=
+      if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)grid_scan_smem<R, C>(C::kNB)) !=
           cudaSuccess)
         return COX_ECUDA;
-      g = persistent_grid(k, C::kThreads, grid_scan_smem<R>(C::kNB), 1 << 30);
+      g = persistent_grid(k, C::kThreads, grid_scan_smem<R, C>(C::kNB), 1 << 30);
     }
-    // as many buffers as give every CTA work: a short array's tiles spread
-    // over the CTAs instead of queueing in the first ones
+    // as many buffers as give every CTA work: an array's tiles spread over the
+    // CTAs instead of queueing in the first ones; one that fits the buffers is
+    // loaded all at once
     const int64_t ctas = ntiles < g ? ntiles : g;
     const int nb = (int)std::min<int64_t>(C::kNB, (ntiles + ctas - 1) / ctas);
-    // an array that fits the buffers is loaded all at once
     const int flight = ntiles <= ctas * nb ? nb : C::kFlight;
-    k<<<(unsigned)ctas, C::kThreads, grid_scan_smem<R>(nb), st>>>(
-        tin, tout, in, out, n, static_cast<unsigned*>(ws),
-        reinterpret_cast<uint64_t*>(static_cast<char*>(ws) + kScanWsHeader), ntiles, excl, nb, flight, spin_limit(),
-        device_status_word());
+    k<<<(unsigned)ctas, C::kThreads, grid_scan_smem<R, C>(nb), st>>>(tin, tout, in, out, n, ticket, agg, ntiles, excl,
+                                                                     nb, flight, spin_limit(), device_status_word());
     return launch_status();
   }
   constexpr int TILE = grid_scan_tile<R>();

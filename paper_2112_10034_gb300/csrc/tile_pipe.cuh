@@ -82,21 +82,27 @@ struct PipePos {
   __device__ uint32_t parity() const { return round & 1u; }
 };
 
-// Runs the pipeline on a CTA of NW + 3 warps, nb <= NB of the buffers in use
-// and at most `flight` loads in flight.  `op` provides, with `slot` the tile's
+// Runs the pipeline on a CTA of NG * NW + 3 warps, nb <= NB of the buffers in
+// use and at most `flight` loads in flight.  The workers are NG groups of NW
+// warps, group g taking every NG-th of the CTA's tiles from its g-th on.  `op` provides, with `slot` the tile's
 // buffer:
 //   load(slot, tile)     one thread: starts the copies that complete full[slot]
 //   fold(slot, tile)     each worker warp: its part of the tile's aggregate
 //   publish(slot, tile)  the last worker warp to fold it
-//   prefix(slot, tile, abort)  the prefix warp: leaves the tile's prefix in
+//   prefix(slot, tile, limit, abort)  the prefix warp: leaves the tile's prefix in
 //                        shared memory; false: gave up
 //   finish(slot, tile)   each worker warp: its part of the results
 //   store(slot, tile)    one thread: copies out of the buffer; returns when
 //                        they have read it
-template <int NB, int NW, class Op>
+template <int NB, int NW, int NG, class Op>
 __device__ __forceinline__ void tile_pipe(PipeShared<NB>& ps, Op& op, int nb, int flight, int64_t ntiles,
                                           unsigned* ticket, uint32_t limit, unsigned* status) {
   const int warp = threadIdx.x >> 5, lane = lane_id();
+  // Worker groups in use: a divisor of nb, so that a slot's tiles belong to
+  // one group, which has finished the slot's last tile before it asks for the
+  // next (a parity can only be told from the one before).
+  int ng = min(NG, nb);
+  while (nb % ng) --ng;
   if (threadIdx.x == 0) {
     for (int b = 0; b < NB; ++b) {
       mbar_init(ps.full + b, 1);
@@ -116,7 +122,7 @@ __device__ __forceinline__ void tile_pipe(PipeShared<NB>& ps, Op& op, int nb, in
       atomicOr(status, (unsigned)kDevTimeout);
     }
   };
-  if (warp == NW) {  // ------------------------------------------- loader
+  if (warp == NG * NW) {  // ------------------------------------------- loader
     PipePos at, ahead;  // the next tile; the one `flight` before it
     bool ok = true;
     int64_t k = 0;
@@ -145,6 +151,14 @@ __device__ __forceinline__ void tile_pipe(PipeShared<NB>& ps, Op& op, int nb, in
       if (!more) break;
       at.next(nb);
     }
+    for (int i = 1; ok && i < ng; ++i) {  // the other groups hear of the end on the slots after
+      at.next(nb);
+      if (k + i >= nb) ok = pipe_wait(ps, ps.free + at.slot, at.parity() ^ 1u, limit);
+      if (ok && lane == 0) {
+        ps.tile[at.slot] = -1;
+        mbar_arrive(ps.full + at.slot);
+      }
+    }
     if (ok) return;
     give_up();
     if (lane == 0)  // copies in flight land before the CTA ends
@@ -153,13 +167,13 @@ __device__ __forceinline__ void tile_pipe(PipeShared<NB>& ps, Op& op, int nb, in
     __syncwarp();
     return;
   }
-  if (warp == NW + 2) {  // --------------------------------------- prefix
+  if (warp == NG * NW + 2) {  // --------------------------------------- prefix
     for (PipePos at;; at.next(nb)) {
       if (!pipe_wait(ps, ps.full + at.slot, at.parity(), limit)) break;
       const int64_t tile = ps.tile[at.slot];
       if (tile < 0) return;
       if (!pipe_wait(ps, ps.folded + at.slot, at.parity(), limit)) break;
-      const bool ok = op.prefix(at.slot, tile, &ps.abort);
+      const bool ok = op.prefix(at.slot, tile, limit, &ps.abort);
       __syncwarp();
       if (!ok) break;
       if (lane == 0) mbar_arrive(ps.pref + at.slot);
@@ -167,7 +181,7 @@ __device__ __forceinline__ void tile_pipe(PipeShared<NB>& ps, Op& op, int nb, in
     give_up();
     return;
   }
-  if (warp == NW + 1) {  // ---------------------------------------- store
+  if (warp == NG * NW + 1) {  // ---------------------------------------- store
     for (PipePos at;; at.next(nb)) {
       if (!pipe_wait(ps, ps.full + at.slot, at.parity(), limit)) break;
       const int64_t tile = ps.tile[at.slot];
@@ -183,8 +197,14 @@ __device__ __forceinline__ void tile_pipe(PipeShared<NB>& ps, Op& op, int nb, in
     return;
   }
   // ---------------------------------------------------------- workers
+  const int group = warp / NW;
+  if (group >= ng) return;
   PipePos f, p;  // the next tile to fold, to finish
-  int held = 0;  // folded, not finished
+  for (int i = 0; i < group; ++i) {
+    f.next(nb);
+    p.next(nb);
+  }
+  int held = 0;  // slots from p to f
   bool ended = false;
   uint32_t spin = 0;
   for (;;) {
@@ -211,8 +231,8 @@ __device__ __forceinline__ void tile_pipe(PipeShared<NB>& ps, Op& op, int nb, in
           mbar_arrive(ps.folded + f.slot);
         }
       }
-      ++held;
-      f.next(nb);
+      held += ng;
+      for (int i = 0; i < ng; ++i) f.next(nb);
       continue;
     }
     if (held) {
@@ -221,8 +241,8 @@ __device__ __forceinline__ void tile_pipe(PipeShared<NB>& ps, Op& op, int nb, in
         op.finish(p.slot, ps.tile[p.slot]);
         __syncwarp();
         if (lane == 0) mbar_arrive(ps.done + p.slot);
-        --held;
-        p.next(nb);
+        held -= ng;
+        for (int i = 0; i < ng; ++i) p.next(nb);
         continue;
       }
     } else if (ended) {

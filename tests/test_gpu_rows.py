@@ -65,22 +65,24 @@ def _grid_scan(cox, src, n, op, dt, comp, excl):  # noqa: F811
     return out[:n]
 
 
-GRID_TILE = {0: 6144, 1: 8192}  # elements per tile: 32-bit values, compensated pairs
+GRID_TILE = {0: 6144, 1: 8192}  # elements per tile of the pipeline: 32-bit values, compensated pairs
 GRID_BUFS = {0: 9, 1: 6}        # tiles a CTA keeps
+SHORT_TILE = 8192               # of the short form, eight per SM at most
 
 
-@pytest.mark.parametrize("where", ["row", "tile", "grid", "buffers"])
+@pytest.mark.parametrize("where", ["row", "tile", "short", "buffers"])
 @pytest.mark.parametrize("delta", [-33, -1, 0, 1, 32])
 @pytest.mark.parametrize("dt,op,comp", [(o.I32, o.SUM, 0), (o.U32, o.MAX, 0), (o.I32, o.XOR, 0), (o.F32, o.MIN, 0),
                                         (o.F32, o.SUM, 1)])
 def test_grid_scan_pipeline_equals_the_general_kernel(cox, where, delta, dt, op, comp):  # noqa: F811
-    """Aligned arrays (the tile pipeline) against the same values 4 bytes off
+    """Aligned arrays (the short form, the tile pipeline) against the same values 4 bytes off
     (the general kernel): whole numbers bit for bit, compensated sums to one
     rounding of the output (2^-24) on either side."""
     import torch
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     t = GRID_TILE[comp]
-    n = {"row": 64, "tile": 3 * t, "grid": sms * t, "buffers": sms * GRID_BUFS[comp] * t}[where] + delta
+    n = {"row": 64, "tile": 3 * SHORT_TILE, "short": 8 * sms * SHORT_TILE,
+         "buffers": sms * (GRID_BUFS[comp] + 4) * t}[where] + delta
     g = torch.Generator(device="cuda")
     g.manual_seed(n + op)
     x = torch.randn(n, generator=g, device="cuda").view(torch.int32) if dt == o.F32 else \
