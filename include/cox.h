@@ -159,11 +159,10 @@ cox_status cox_tile_scan(cox_op op, cox_dtype dt, int width, int block_dim, cons
  * with warp shuffle scans and a scan of the warp totals, and uniform_add adds
  * each block's prefix (Table 1).  BLOCK scope does the first part on blocks
  * of block_dim elements; GRID scope chains tiles (16-byte aligned arrays:
- * 8192 elements by TMA, 16384 for compensated sums; other layouts: 16384,
- * 8192 compensated) with the decoupled look-back of cox_ballot_compact: in a
- * tile every warp scans its rows of 32 elements by shfl_up, carries row
- * totals across its rows, the warp totals are scanned, the tile publishes
- * its aggregate, looks back for its prefix and adds it.
+ * 6144 or 8192 elements by TMA; other layouts: 16384, 8192 compensated): in a
+ * tile every warp scans its rows of 32 elements, carries row totals across its
+ * rows, the warp totals are scanned, the tile publishes its aggregate, and its
+ * prefix -- the fold of all earlier tiles' aggregates -- is added.
  *   d_out[i] = x[s] op ... op x[i] (inclusive) or x[s] op ... op x[i-1] with
  *   the identity at i = s (exclusive), s = the first index of i's block
  *   (BLOCK) or 0 (GRID).
@@ -171,12 +170,11 @@ cox_status cox_tile_scan(cox_op op, cox_dtype dt, int width, int block_dim, cons
  *   exclusive: 0 or 1.
  *   d_workspace: GRID only, cox_scan_workspace() bytes, 16-byte aligned,
  *   zeroed by the call (cudaMemsetAsync).  Not shared across concurrent calls.
- * Integer results are exact.  GRID fp32 results take each tile's prefix in
- * the order its look-back found the predecessors' values, so their last bits
- * may differ from run to run (within the stated tolerance); a compensated
- * prefix passes between tiles with its error word rounded to 21 mantissa
- * bits (about 2^-46 of the sum).  BLOCK results are reproducible.
- * Look-back waits are bounded as in cox_ballot_compact.
+ * Integer results are exact.  GRID fp32 results take each tile's prefix in the
+ * order in which the earlier aggregates were found, so their last bits may
+ * differ from run to run (within the stated tolerance).  BLOCK results are
+ * reproducible.
+ * Waits for aggregates are bounded as in cox_ballot_compact.
  */
 cox_status cox_scan(cox_op op, cox_dtype dt, cox_scope scope, int block_dim, const void* d_in, void* d_out,
                     int64_t n, unsigned flags, int exclusive, void* d_workspace, size_t workspace_bytes,
@@ -319,16 +317,16 @@ size_t cox_integral_image_workspace(int64_t batch, int64_t height, int64_t width
  *   unless flags has COX_F_WS_READY, in which case the caller guarantees those
  *   bytes are zero.  Not shared across concurrent calls.
  *   flags: 0 or COX_F_WS_READY.
- * Tiles of 8192 keys go round-robin to the CTAs of one cooperative launch
- * (256 threads each, whatever block_dim: the result does not depend on the
- * block size, which is only validated); each tile's look-back polls its
- * predecessors' descriptors.  A poll that exceeds the spin limit
- * (cox_set_spin_limit) gives up: the tile publishes a zero prefix, writes
+ * Tiles of 8192 keys (whatever block_dim: the result does not depend on the
+ * block size, which is only validated) are handed to the CTAs by an atomic
+ * ticket in the workspace's header; a tile's prefix is the sum of all earlier
+ * tiles' published counts.  A poll for a count that exceeds the spin limit
+ * (cox_set_spin_limit) gives up: the CTA stops, its unfinished tiles write
  * nothing, and COX_ETIMEOUT is recorded for cox_device_status().  With
  * COX_F_WS_READY, a descriptor word whose two top bits are both set is
  * "withheld": it reads as not yet published, and no publish overwrites it
  * (a way to test that the waits end).  Every write stays inside d_out[0, n)
- * and d_count.  COX_ECUDA if the cooperative launch is refused.
+ * and d_count.  COX_ECUDA if the launch is refused.
  */
 cox_status cox_ballot_compact(cox_dtype dt, int width, int block_dim, const void* d_keys, int64_t n,
                               int64_t threshold, void* d_out, int64_t* d_count, void* d_workspace,

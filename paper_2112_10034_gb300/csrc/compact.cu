@@ -1,23 +1,21 @@
 // cox_ballot_compact: stable stream compaction from warp ballots.
 //
-// A cooperative launch of 256-thread CTAs (three per SM, whatever the
-// caller's block size: the result does not depend on it); CTA c takes tiles
-// c, c + G, ... of 8192 keys (32 KB).  Each CTA keeps two tiles in shared
-// memory: one is worked on while the next arrives by a TMA bulk copy (plain
-// loads for a ragged or unaligned tile), so the copies stay in flight while
-// tiles wait on their look-backs.  In a tile (compact_tile.cuh):
-//   compact every warp compacts its 1024 keys in place in one pass: per
-//           chunk of 128 keys, b = __ballot_sync(keep) for each of a lane's
-//           four key slots, rank = kept keys before the chunk +
-//           popc(b & lanemask_lt) over the slots + kept keys before it in
-//           the lane;
-//   scan    warp 0 scans the 8 warp counts and publishes the tile's count
-//           for the look-back;
-//   prefix  warp 0's decoupled look-back;
-//   out     every warp copies its kept keys to out[prefix + offset ..].
+// Tiles of 8192 keys (32 KB) arrive by TMA bulk copies (plain loads for a
+// ragged or unaligned tile) and go through the tile pipeline (tile_pipe.cuh;
+// short arrays: one tile per CTA).  In a tile, by eight warps:
+//   fold    every warp compacts its 1024 keys in place in one pass
+//           (compact_tile.cuh): per chunk of 128 keys, b =
+//           __ballot_sync(keep) for each of a lane's four key slots, rank =
+//           kept keys before the chunk + popc(b & lanemask_lt) over the slots
+//           + kept keys before it in the lane;
+//   publish the scan of the 8 warp counts; the tile's count;
+//   prefix  the counts of all earlier tiles;
+//   finish  every warp copies its kept keys to out[prefix + offset ..].
+#include <algorithm>
 #include <mutex>
 
 #include "compact_tile.cuh"
+#include "tile_pipe.cuh"
 
 namespace cox {
 
@@ -25,113 +23,208 @@ constexpr int kCompactThreads = 256;
 constexpr int kCompactNW = kCompactThreads / 32;
 constexpr int kCompactReg = 1024;                            // keys per warp
 constexpr int64_t kCompactTile = kCompactNW * kCompactReg;  // 8192 keys
-constexpr int kCompactBufs = 2;                              // tiles in shared memory per CTA
+constexpr uint32_t kCompactTileBytes = (uint32_t)kCompactTile * 4;
+// Shape of the pipeline, one CTA per SM: six tiles, two groups of eight worker
+// warps, three loads in flight.  2^28 keys at d = 0.1 / 0.5 / 0.9: 249 / 283 /
+// 323 us (4740 / 5700 / 6310 GB/s); one group 344 / 367 / 394, three 252 / 283
+// / 322 (the workers' passes over the keys, then the tile's way through shared
+// memory, bound it).  The cooperative kernel before it, two tiles per CTA and a
+// look-back per tile, ran 271 / 326 / 372 us, with this tile body 273 / 327 /
+// 371.
+constexpr int kCompactNB = 6;      // tiles in shared memory
+constexpr int kCompactNG = 2;      // groups of eight worker warps
+constexpr int kCompactFlight = 3;  // loads in flight
+// Up to this many tiles per SM every tile has a CTA of its own (six fit).
+// 10^6 keys at d = 0.5 8.3 us against 10.3 through the pipeline, 2^22 13.8
+// against 17.9, 2^23 22.4 against 22.0, 2^24 32.3 against 30.2.
+constexpr int kCompactShortTiles = 6;
+constexpr int kCompactPipeThreads = (kCompactNG * kCompactNW + 3) * 32;
 
-// A cooperative launch (all CTAs co-resident) of G CTAs, three per SM; CTA c
-// takes tiles c, c + G, c + 2G, ... in turn, with the next tile's TMA bulk
-// copy in flight while it works on the current one.  Per tile: every warp
-// compacts its 1024 keys in place, warp 0 scans the warp counts, publishes
-// the tile's count and looks back for its prefix, every warp copies its kept
-// keys to out[prefix + the warps before it ..], and the freed buffer starts
-// loading the tile after next.  A CTA works on its tiles in increasing order
-// and all CTAs run at once, so the lowest unfinished tile always has every
-// predecessor finished: every look-back wait ends (each is bounded all the
-// same).
-template <bool SIGNED>
-__global__ void __launch_bounds__(kCompactThreads, 3) k_ballot_compact(const uint32_t* __restrict__ keys, int64_t n,
-                                                         int64_t thr, uint32_t* __restrict__ out,
-                                                         int64_t* __restrict__ d_count, uint64_t* desc,
-                                                         int64_t ntiles, uint32_t limit, unsigned* status, int vec) {
-  extern __shared__ __align__(16) uint32_t smem[];
-  const int64_t TILE = kCompactTile;
-  uint32_t* wcnt = smem + kCompactBufs * TILE;  // warp counts, then offsets
-  uint64_t* bar = reinterpret_cast<uint64_t*>(wcnt + kCompactWsWords);
-  __shared__ int64_t s_prefix;
-  __shared__ uint32_t s_total;
-  __shared__ int s_bad;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int region = warp * kCompactReg;
-  const unsigned lt = lanemask_lt();
-  const LeRule rule = le_rule<SIGNED>(thr);
-  const int64_t G = gridDim.x;
-  // tile k of this CTA: blockIdx.x + k G, in buffer k % kCompactBufs
-  auto bulk = [&](int64_t tile) { return vec && (tile + 1) * TILE <= n; };
-  auto issue = [&](int64_t k) {  // thread 0: start loading this CTA's tile k
-    const int64_t tile = blockIdx.x + k * G;
-    if (tile < ntiles && bulk(tile)) {
-      uint64_t* b = bar + (k % kCompactBufs);
-      mbar_arrive_expect_tx(b, (uint32_t)(TILE * 4));
-      tma_load_1d(smem + (k % kCompactBufs) * TILE, keys + tile * TILE, (uint32_t)(TILE * 4), b);
+template <int NB>
+struct CompactShared {
+  PipeShared<NB> pipe;
+  uint32_t cnt[NB][kCompactNW];   // a warp's kept keys
+  uint32_t off[NB][kCompactNW];   // kept keys of the tile's warps before it
+  uint32_t total[NB];
+  int64_t prefix[NB];
+};
+
+// A published count: flag A (desc_missing tells flags 0 and 3 apart from it).
+__device__ __forceinline__ bool count_there(uint64_t d) { return !desc_missing(d); }
+
+template <bool SIGNED, int NB>
+struct CompactOp {
+  const uint32_t* keys;
+  int64_t n;
+  LeRule rule;
+  uint32_t* out;
+  int64_t* d_count;
+  uint64_t* desc;
+  int64_t ntiles;
+  int vec;
+  uint32_t* bufs;
+  CompactShared<NB>* sh;
+  static constexpr int kWin = 8;  // 32-tile rows per poll of the walk
+  int64_t cur = 0, run = 0, base = 0;  // the prefix warp's walk (as AggWalk of the grid scan)
+
+  __device__ uint32_t* buf(int slot) const { return bufs + (size_t)slot * kCompactTile; }
+  __device__ bool bulk(int64_t tile) const { return vec && (tile + 1) * kCompactTile <= n; }
+
+  __device__ void load(int slot, int64_t tile) const {
+    uint64_t* bar = sh->pipe.full + slot;
+    if (bulk(tile)) {
+      mbar_arrive_expect_tx(bar, kCompactTileBytes);
+      tma_load_1d(buf(slot), keys + tile * kCompactTile, kCompactTileBytes, bar);
+    } else {
+      mbar_arrive(bar);
     }
-  };
+  }
+  __device__ void fold(int slot, int64_t tile) const {
+    const int lane = lane_id(), warp = (threadIdx.x >> 5) % kCompactNW, region = warp * kCompactReg;
+    uint32_t* b = buf(slot);
+    const int valid = (int)min(kCompactTile, n - tile * kCompactTile);
+    if (!bulk(tile)) {
+      for (int i = region + lane; i < min(valid, region + kCompactReg); i += 32) b[i] = keys[tile * kCompactTile + i];
+      __syncwarp();
+    }
+    const uint32_t kept =
+        compact_region<SIGNED, kCompactReg>(b, region, lane, lanemask_lt(), valid, valid == (int)kCompactTile, rule);
+    if (lane == 0) sh->cnt[slot][warp] = kept;
+  }
+  __device__ void publish(int slot, int64_t tile) const {
+    const int lane = lane_id();
+    const uint32_t c = lane < kCompactNW ? sh->cnt[slot][lane] : 0u;
+    uint32_t incl = c;
+#pragma unroll
+    for (int d = 1; d < kCompactNW; d <<= 1) {
+      const uint32_t u = __shfl_up_sync(kFull, incl, d);
+      if (lane >= d) incl += u;
+    }
+    if (lane < kCompactNW) sh->off[slot][lane] = incl - c;
+    if (lane == kCompactNW - 1) {
+      sh->total[slot] = incl;
+      desc_raise(desc + tile, kFlagA | incl);
+    }
+  }
+  __device__ bool prefix(int slot, int64_t tile, uint32_t limit, volatile int* abort) {
+    const int lane = lane_id();
+    uint32_t polls = 0;
+    while (cur < tile) {
+      uint64_t w[kWin];
+#pragma unroll
+      for (int v = 0; v < kWin; ++v) {
+        const int64_t t = cur + v * 32 + lane;
+        w[v] = t < tile ? ld_relaxed_u64(desc + t) : 0;
+      }
+      uint32_t part = 0;
+      int step = 0;
+#pragma unroll
+      for (int v = 0; v < kWin; ++v) {
+        if (step != v * 32) break;  // (a gap in an earlier row)
+        const unsigned there = __ballot_sync(kFull, count_there(w[v]));
+        const int k = there == kFull ? 32 : __ffs(~there) - 1;
+        if (lane < k) part += (uint32_t)w[v];
+        step += k;
+      }
+      if (step) {
+        run += __reduce_add_sync(kFull, part);
+        cur += step;
+        polls = 0;
+        continue;
+      }
+      if (++polls > limit || __any_sync(kFull, *abort)) return false;
+      __nanosleep(polls > 64 ? 200 : 20);
+    }
+    if (lane == 0) sh->prefix[slot] = run;
+    return true;
+  }
+  __device__ void finish(int slot, int64_t tile) const {
+    const int lane = lane_id(), warp = (threadIdx.x >> 5) % kCompactNW;
+    const int64_t prefix = sh->prefix[slot];
+    const uint32_t total = sh->total[slot];
+    if (prefix + (int64_t)total <= n) {
+      uint32_t* dst = out + prefix + sh->off[slot][warp];
+      const uint32_t* src = buf(slot) + warp * kCompactReg;
+      const int kept = (int)sh->cnt[slot][warp];
+#pragma unroll 4
+      for (int i = lane; i < kept; i += 32) dst[i] = src[i];
+      if (tile == ntiles - 1 && warp == 0 && lane == 0) *d_count = prefix + total;
+    }
+    fence_proxy_async_smem();  // before the bulk copy that refills the buffer
+  }
+  __device__ void store(int, int64_t) const {}
+};
+
+template <bool SIGNED>
+__global__ void __launch_bounds__(kCompactPipeThreads, 1)
+    k_ballot_compact(const uint32_t* __restrict__ keys, int64_t n, int64_t thr, uint32_t* __restrict__ out,
+                     int64_t* __restrict__ d_count, unsigned* ticket, uint64_t* desc, int64_t ntiles, int nb,
+                     int flight, uint32_t limit, unsigned* status, int vec) {
+  extern __shared__ __align__(16) uint32_t smem[];
+  auto* sh = reinterpret_cast<CompactShared<kCompactNB>*>(smem + (size_t)nb * kCompactTile);
+  CompactOp<SIGNED, kCompactNB> op{keys, n, le_rule<SIGNED>(thr), out, d_count, desc, ntiles, vec, smem, sh};
+  tile_pipe<kCompactNB, kCompactNW, kCompactNG>(sh->pipe, op, nb, flight, ntiles, ticket, limit, status);
+}
+
+// Short arrays, whose tiles are resident at once: one tile per CTA, several
+// CTAs per SM, the prefix gathered by all warps together.
+template <bool SIGNED>
+__global__ void __launch_bounds__(kCompactThreads, 6)
+    k_ballot_compact_short(const uint32_t* __restrict__ keys, int64_t n, int64_t thr, uint32_t* __restrict__ out,
+                           int64_t* __restrict__ d_count, unsigned* ticket, uint64_t* desc, int64_t ntiles,
+                           uint32_t limit, unsigned* status, int vec) {
+  extern __shared__ __align__(16) uint32_t smem[];
+  auto* sh = reinterpret_cast<CompactShared<1>*>(smem + kCompactTile);
+  __shared__ int64_t s_tile;
+  __shared__ uint32_t s_part[kCompactNW];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  CompactOp<SIGNED, 1> op{keys, n, le_rule<SIGNED>(thr), out, d_count, desc, ntiles, vec, smem, sh};
   if (tid == 0) {
-    for (int b = 0; b < kCompactBufs; ++b) mbar_init(bar + b, 1);
+    mbar_init(sh->pipe.full, 1);
     mbar_init_fence();
-    for (int k = 0; k < kCompactBufs; ++k) issue(k);
+    const int64_t t = (int64_t)atomicAdd(ticket, 1u);
+    op.load(0, t);
+    s_tile = t;
   }
   __syncthreads();
-  for (int64_t k = 0;; ++k) {
-    const int64_t tile = blockIdx.x + k * G;
-    if (tile >= ntiles) break;
-    uint32_t* buf = smem + (k % kCompactBufs) * TILE;
-    const int64_t base = tile * TILE;
-    const int valid = (int)min(TILE, n - base);
-    // ---- the tile in shared memory
-    if (bulk(tile)) {
-      const uint32_t parity = (uint32_t)((k / kCompactBufs) & 1);
-      const bool ok = mbar_wait_bounded(bar + (k % kCompactBufs), parity, limit);
-      if (__syncthreads_or(!ok)) {  // a copy did not land in time: record it, let the copies in flight land, stop
-        if (tid == 0) {
-          atomicOr(status, (unsigned)kDevTimeout);
-          for (int64_t j = k; j < k + kCompactBufs; ++j)
-            if (blockIdx.x + j * G < ntiles && bulk(blockIdx.x + j * G))
-              mbar_wait_bounded(bar + (j % kCompactBufs), (uint32_t)((j / kCompactBufs) & 1), limit);
-          for (int64_t t = tile; t < ntiles; t += G) desc_raise(desc + t, kFlagP);  // successors end
-        }
+  const int64_t tile = s_tile;
+  if (__syncthreads_or(!mbar_wait_bounded(sh->pipe.full, 0u, limit))) {
+    if (tid == 0) {
+      atomicOr(status, (unsigned)kDevTimeout);
+      mbar_wait_bounded(sh->pipe.full, 0u, limit);
+    }
+    return;
+  }
+  op.fold(0, tile);
+  __syncthreads();
+  if (warp == 0) op.publish(0, tile);
+  uint32_t part = 0;
+  bool ok = true;
+  for (int64_t t = tid; ok && t < tile; t += kCompactThreads) {
+    uint64_t d;
+    for (uint32_t polls = 0; !count_there(d = ld_relaxed_u64(desc + t)); ++polls) {
+      if (polls > limit) {
+        ok = false;
         break;
       }
-    } else {
-      for (int i = tid; i < valid; i += kCompactThreads) buf[i] = keys[base + i];
-      __syncthreads();
+      __nanosleep(polls > 64 ? 200 : 20);
     }
-    // ---- every warp compacts its region in place
-    const uint32_t kept = compact_region<SIGNED, kCompactReg>(buf, region, lane, lt, valid, valid == (int)TILE, rule);
-    if (lane == 0) wcnt[warp] = kept;
-    __syncthreads();
-    // ---- count, look-back, offsets
-    if (warp == 0) {
-      const uint32_t wc = lane < kCompactNW ? wcnt[lane] : 0u;
-      uint32_t incl = wc;
-#pragma unroll
-      for (int d = 1; d < kCompactNW; d <<= 1) {
-        const uint32_t u = __shfl_up_sync(kFull, incl, d);
-        if (lane >= d) incl += u;
-      }
-      const uint32_t total = __shfl_sync(kFull, incl, kCompactNW - 1);
-      if (lane < kCompactNW) wcnt[32 + lane] = incl - wc;  // exclusive offsets
-      if (lane == 0) publish_count(desc, tile, ntiles, total);
-      bool gave_up;
-      const int64_t prefix = look_back(desc, tile, ntiles, total, limit, status, gave_up);
-      if (lane == 0) {
-        s_prefix = prefix;
-        s_total = total;
-        s_bad = gave_up;
-      }
-    }
-    __syncthreads();
-    // ---- copy-out
-    const int64_t prefix = s_prefix;
-    if (!s_bad && prefix + (int64_t)s_total <= n) {
-      uint32_t* dst = out + prefix + wcnt[32 + warp];
-      const uint32_t* src = buf + region;
-#pragma unroll 4
-      for (int i = lane; i < (int)kept; i += 32) dst[i] = src[i];
-      if (tile == ntiles - 1 && tid == 0) *d_count = prefix + s_total;
-    }
-    fence_proxy_async_smem();  // this thread's accesses to the buffer, before the bulk copy that refills it
-    __syncthreads();
-    if (tid == 0) issue(k + kCompactBufs);
+    part += (uint32_t)d;
   }
+  __syncwarp();
+  part = __reduce_add_sync(kFull, part);
+  if (lane == 0) s_part[warp] = part;
+  if (__syncthreads_or(!ok)) {
+    if (tid == 0) atomicOr(status, (unsigned)kDevTimeout);
+    return;
+  }
+  if (tid == 0) {
+    int64_t p = 0;
+    for (int k = 0; k < kCompactNW; ++k) p += s_part[k];
+    sh->prefix[0] = p;
+  }
+  __syncthreads();
+  op.finish(0, tile);
 }
 
 }  // namespace cox
@@ -161,31 +254,40 @@ extern "C" cox_status cox_ballot_compact(cox_dtype dt, int width, int block_dim,
   if (!(flags & COX_F_WS_READY) && cudaMemsetAsync(d_workspace, 0, need, st) != cudaSuccess) return COX_ECUDA;
   const int64_t tile = kCompactTile;
   const int64_t ntiles = (n + tile - 1) / tile;
-  const size_t smem = ((size_t)kCompactBufs * tile + kCompactWsWords) * sizeof(uint32_t) + kCompactBufs * sizeof(uint64_t);
+  unsigned* ticket = static_cast<unsigned*>(d_workspace);  // in the header, zero like the descriptors
   uint64_t* desc = reinterpret_cast<uint64_t*>(static_cast<char*>(d_workspace) + kCompactWsHeader);
   const int vec = aligned16(d_keys);
+  const uint32_t* keys = static_cast<const uint32_t*>(d_keys);
+  uint32_t* outp = static_cast<uint32_t*>(d_out);
+  if (ntiles <= (int64_t)kCompactShortTiles * sm_count()) {
+    const size_t smem = kCompactTileBytes + sizeof(CompactShared<1>);
+    auto go = [&](auto kern) {
+      kern<<<(unsigned)ntiles, kCompactThreads, smem, st>>>(keys, n, threshold, outp, d_count, ticket, desc, ntiles,
+                                                            spin_limit(), device_status_word(), vec);
+      return launch_status();
+    };
+    return dt == COX_I32 ? go(k_ballot_compact_short<true>) : go(k_ballot_compact_short<false>);
+  }
+  auto smem = [](int nb) { return (size_t)nb * kCompactTileBytes + sizeof(CompactShared<kCompactNB>); };
   auto launch = [&](auto kern, int* grid) {
     int& g = grid[device_index()];
     if (g == 0) {
-      if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+      if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem(kCompactNB)) !=
+          cudaSuccess)
         return COX_ECUDA;
-      g = persistent_grid(kern, kCompactThreads, smem, 1 << 30);
+      g = persistent_grid(kern, kCompactPipeThreads, smem(kCompactNB), 1 << 30);
     }
+    // as many buffers as give every CTA work, in whole rounds of the groups
     const int64_t ctas = ntiles < g ? ntiles : g;
-    const uint32_t* keys = static_cast<const uint32_t*>(d_keys);
-    uint32_t* outp = static_cast<uint32_t*>(d_out);
-    uint32_t limit = spin_limit();
-    unsigned* status = device_status_word();
-    void* args[] = {(void*)&keys, (void*)&n, (void*)&threshold, (void*)&outp, (void*)&d_count, (void*)&desc,
-                    (void*)&ntiles, (void*)&limit, (void*)&status, (void*)&vec};
-    if (cudaLaunchCooperativeKernel((const void*)kern, dim3((unsigned)ctas), dim3(kCompactThreads), args, smem, st) !=
-        cudaSuccess) {
-      cudaGetLastError();
-      return COX_ECUDA;
-    }
-    return COX_OK;
+    int nb = (int)std::min<int64_t>(kCompactNB, (ntiles + ctas - 1) / ctas);
+    if (nb > kCompactNG) nb = (nb + kCompactNG - 1) / kCompactNG * kCompactNG;
+    const int flight = ntiles <= ctas * nb ? nb : kCompactFlight;
+    kern<<<(unsigned)ctas, kCompactPipeThreads, smem(nb), st>>>(keys, n, threshold, outp, d_count, ticket, desc,
+                                                                ntiles, nb, flight, spin_limit(),
+                                                                device_status_word(), vec);
+    return launch_status();
   };
-  static int grid_s[kMaxDevices], grid_u[kMaxDevices];  // co-resident grids, per device
+  static int grid_s[kMaxDevices], grid_u[kMaxDevices];  // resident CTAs, per device
   return dt == COX_I32 ? launch(k_ballot_compact<true>, grid_s) : launch(k_ballot_compact<false>, grid_u);
 }
 

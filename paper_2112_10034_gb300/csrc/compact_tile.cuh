@@ -216,59 +216,38 @@ __device__ __forceinline__ bool keep_le(uint32_t k, uint32_t tm) {
 }
 
 // The tile body runs NW warps per CTA on a tile of NW * 2048 keys: each warp
-// owns a region of 2048 keys, which it reads as four sub-runs of 512 (lane l
-// holds keys 128q + 4l .. 128q + 4l + 3 of a sub-run, q = 0..3:
-// conflict-free 128-bit shared loads).
+// owns a region of 2048 keys, which it reads as four sub-runs of 512.
 constexpr int kCompactRegion = 2048;  // keys per warp
 constexpr int kCompactWsWords = 2 * 32;  // shared words the tile body needs (counts, offsets), any NW <= 32
 
 // One sub-run of a warp's region, compacted in place to the front of the
-// region.  Per chunk q and key slot k every lane votes b = __ballot_sync(keep);
-// a kept key's rank in the region is
-//   kept keys of earlier sub-runs and chunks + sum_k' popc(b_k' & lanes below)
-//     + kept keys before it in its lane,
-// i.e. its position in input order.  Ranks never exceed the key's own index,
-// so the writes only reach keys every lane has already loaded (the
-// __syncwarp after the loads orders them).  Returns the sub-run's count.
+// region: 16 rows of 32 keys, lane l holding key 32 r + l.  Per row every lane
+// votes b = __ballot_sync(keep), and a kept key's rank in the region is
+//   kept keys of earlier rows + popc(b & lanes below),
+// i.e. its position in input order; a row's kept keys go to consecutive words
+// (no bank conflicts).  A row takes about ten warp instructions; lanes holding
+// four consecutive keys each (a quarter of the shared loads, but every rank
+// from four votes) took 18.7.  Ranks never exceed the key's own index, so the
+// writes only reach keys every lane has already loaded (the __syncwarp after
+// the loads orders them).  Returns the sub-run's count.
 template <bool SIGNED, bool FULL>
 __device__ __forceinline__ uint32_t compact_subrun(uint32_t* buf, int region, int sub, int lane, unsigned lt,
                                                    int valid, uint32_t tm, uint32_t kept_before) {
-  const int sb = region + 512 * sub;
-  uint32_t key[4][4];
-  bool kp[4][4];
+  const int i0 = region + 512 * sub + lane;
+  uint32_t key[16];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int i0 = sb + 128 * q + 4 * lane;
-    const uint4 v = *reinterpret_cast<const uint4*>(buf + i0);
-    key[q][0] = v.x; key[q][1] = v.y; key[q][2] = v.z; key[q][3] = v.w;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) kp[q][k] = (FULL || i0 + k < valid) && keep_le<SIGNED>(key[q][k], tm);
-  }
-  uint32_t below[4], total[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    below[q] = 0;
-    total[q] = 0;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const unsigned b = __ballot_sync(kFull, kp[q][k]);
-      below[q] += __popc(b & lt);
-      total[q] += __popc(b);
-    }
-  }
+  for (int r = 0; r < 16; ++r) key[r] = buf[i0 + 32 * r];
   __syncwarp();  // every lane's loads of this sub-run before any write into it
-  uint32_t chunk_base = kept_before;
+  uint32_t* o = buf + region + kept_before;
+  uint32_t kept = 0;
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    uint32_t* o = buf + region + chunk_base + below[q];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      if (kp[q][k]) *o = key[q][k];
-      o += kp[q][k];
-    }
-    chunk_base += total[q];
+  for (int r = 0; r < 16; ++r) {
+    const bool keep = (FULL || i0 + 32 * r < valid) && keep_le<SIGNED>(key[r], tm);
+    const unsigned b = __ballot_sync(kFull, keep);
+    if (keep) o[kept + __popc(b & lt)] = key[r];
+    kept += __popc(b);
   }
-  return chunk_base - kept_before;
+  return kept;
 }
 
 // A warp's region of REG keys (a multiple of 512) compacted in place to its

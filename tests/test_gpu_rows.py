@@ -113,3 +113,30 @@ def test_grid_scan_is_reproducible_and_works_in_place(cox):  # noqa: F811
     assert cox.cox_scan(o.SUM, o.I32, o.GRID, 256, x.data_ptr(), x.data_ptr(), n, 0, 0, ws.data_ptr(), ws.numel(),
                         None) == cox.COX_OK
     assert torch.equal(x, want)
+
+
+@pytest.mark.parametrize("d", [0.0, 0.3, 1.0])
+@pytest.mark.parametrize("where,delta", [("tile", -1), ("tile", 0), ("tile", 1), ("short", 0), ("short", 1),
+                                         ("buffers", -511), ("buffers", 3)])
+def test_compaction_forms_agree(cox, where, delta, d):  # noqa: F811
+    """One tile per CTA, the tile pipeline, and both from an unaligned address, against a plain filter."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = {"tile": 3, "short": 6 * sms, "buffers": 13 * sms}[where] * 8192 + delta
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n)
+    full = torch.randint(-2**31, 2**31 - 1, (n + 1,), generator=g, device="cuda", dtype=torch.int32)
+    thr = int(-2**31 + d * 2**32)
+    for keys in (full[:n], full[1:]):
+        for dt in (o.I32, o.U32):
+            out = poisoned(n, torch.int32)
+            cnt = torch.full((1,), -1, dtype=torch.int64, device="cuda")
+            ws = torch.full((cox.cox_ballot_compact_workspace(n, 256),), 0xA5, dtype=torch.uint8, device="cuda")
+            t = thr if dt == o.I32 else thr + 2**31
+            assert cox.cox_ballot_compact(dt, 32, 256, keys.data_ptr(), n, t, out.data_ptr(), cnt.data_ptr(),
+                                          ws.data_ptr(), ws.numel(), 0, None) == cox.COX_OK
+            unsigned = keys.long() & 0xFFFFFFFF
+            want = keys[(keys.long() if dt == o.I32 else unsigned) < t]
+            assert int(cnt.item()) == want.numel() and torch.equal(out[:want.numel()], want)
+            assert bool((out[n:] == POISON).all())
+    assert cox.device_status() == cox.COX_OK
