@@ -578,9 +578,15 @@ cox_status cox_server_poll(cox_server* s, uint64_t ticket, int* done);
 cox_status cox_server_wait(cox_server* s, uint64_t ticket, double timeout_s);
 
 /* Device pointer of a done request's output (valid until release) and its
- * element count (REDUCE 1, SCAN n, COMPACT the kept count, read from the
- * device with a synchronous copy). */
+ * element count (REDUCE 1, SCAN n, COMPACT the kept count, which the kernels
+ * leave in pinned host memory: no copy, no synchronisation). */
 cox_status cox_server_result(cox_server* s, uint64_t ticket, void** d_out, int64_t* count);
+
+/* Copies the first `words` 32-bit words of a done request's output to d_dst on
+ * `stream` (REDUCE: 2, the element and its low word).  COX_EINVAL for a ticket
+ * that is not done or more words than the output's room.  The request may be
+ * released once the copy is done. */
+cox_status cox_server_read(cox_server* s, uint64_t ticket, void* d_dst, int64_t words, void* stream);
 
 /* Frees a done request's arena memory and slot. */
 cox_status cox_server_release(cox_server* s, uint64_t ticket);

@@ -72,6 +72,7 @@ SIGNATURES = {
     "cox_server_poll": (_I, [_P, ctypes.c_uint64, _P]),
     "cox_server_wait": (_I, [_P, ctypes.c_uint64, ctypes.c_double]),
     "cox_server_result": (_I, [_P, ctypes.c_uint64, _P, _P]),
+    "cox_server_read": (_I, [_P, ctypes.c_uint64, _P, _I64, _P]),
     "cox_server_release": (_I, [_P, ctypes.c_uint64]),
     "cox_server_get_stats": (_I, [_P, _P]),
     "cox_server_destroy": (None, [_P]),
@@ -533,17 +534,12 @@ def make_request(kind: int, x, width: int = 32, compensated: bool = False, thres
                        x.numel() if n is None else int(n), int(threshold), x.data_ptr())
 
 
-class _DevView:
-    def __init__(self, ptr, n, typestr):
-        self.__cuda_array_interface__ = {"shape": (int(n),), "typestr": typestr, "data": (int(ptr), False),
-                                         "version": 2}
-
-
 class Server:
     """Continuous-batching request server (cox_server_*) over a device arena."""
 
     def __init__(self, budget_bytes: int, max_requests: int = 1024):
         self.handle = ctypes.c_void_p()
+        self._device = _torch().device("cuda", _torch().cuda.current_device())  # the server's
         _check(lib().cox_server_create(int(budget_bytes), int(max_requests), ctypes.byref(self.handle)),
                "cox_server_create")
         self._keep = {}
@@ -577,16 +573,17 @@ class Server:
     def result(self, ticket: int, req: cox_request):
         """A copy (torch CUDA tensor) of a done request's output."""
         t = _torch()
-        p = ctypes.c_void_p()
-        c = ctypes.c_int64()
-        _check(lib().cox_server_result(self.handle, ticket, ctypes.byref(p), ctypes.byref(c)), "cox_server_result")
-        if req.kind == COX_REQ_REDUCE:
-            n, typ = 2, ("<f4" if req.dt == COX_F32 else "<i4")
+        h = lib()
+        if req.kind == COX_REQ_COMPACT:
+            p = ctypes.c_void_p()
+            c = ctypes.c_int64()
+            _check(h.cox_server_result(self.handle, ticket, ctypes.byref(p), ctypes.byref(c)), "cox_server_result")
+            n = c.value
         else:
-            n, typ = c.value, ("<f4" if req.dt == COX_F32 else "<i4")
-        if n == 0:
-            return t.empty(0, dtype=t.float32 if typ == "<f4" else t.int32, device="cuda")
-        return t.as_tensor(_DevView(p.value, n, typ), device="cuda").clone()
+            n = 2 if req.kind == COX_REQ_REDUCE else req.n
+        out = t.empty(n, dtype=t.float32 if req.dt == COX_F32 else t.int32, device=self._device)
+        _check(h.cox_server_read(self.handle, ticket, out.data_ptr(), n, _stream(self._device)), "cox_server_result")
+        return out
 
     def release(self, ticket: int) -> None:
         _check(lib().cox_server_release(self.handle, ticket), "cox_server_release")

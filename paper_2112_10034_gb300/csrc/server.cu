@@ -60,6 +60,7 @@ struct ReqDesc {
   uint32_t* out;
   uint8_t* ws;
   int64_t item0, nitems;
+  int64_t* count;  // COMPACT: receives the kept count (pinned host memory, mapped)
 };
 
 struct BatchHdr {
@@ -355,7 +356,7 @@ __device__ __forceinline__ void serve_body(const ReqDesc* reqs, int nreq, int64_
         for (int i = tid; i < valid; i += blockDim.x) dst[i] = buf[i];
       }
     } else {
-      int64_t* count = reinterpret_cast<int64_t*>(d.ws);
+      int64_t* count = d.count;
       uint64_t* desc = reinterpret_cast<uint64_t*>(d.ws + kAlign);
       if (d.dt == COX_I32)
         compact_big_tile<true, kServeBlock / 32>(buf, valid, d.threshold, d.out, count, desc, c, d.nitems, d.n, limit,
@@ -364,6 +365,8 @@ __device__ __forceinline__ void serve_body(const ReqDesc* reqs, int nreq, int64_
         compact_big_tile<false, kServeBlock / 32>(buf, valid, d.threshold, d.out, count, desc, c, d.nitems, d.n, limit,
                                                   status, wcnt);
     }
+    // the tile that wrote its request's count to host memory: before the mark
+    if (tid == 0 && d.kind == COX_REQ_COMPACT && c == d.nitems - 1) __threadfence_system();
     pending = s_req;  // marked at the top of the next round, once its writes (and bulk store) are done
   }
   // ---- the last tile's mark; the last CTA out zeroes the slot's counters
@@ -510,6 +513,7 @@ struct SReq {
   ReqState state = kQueued;
   size_t off = 0, bytes = 0, out_b = 0, held = 0;
   double t_submit = 0.0, t_ready = 0.0, t_launch = 0.0, t_done = 0.0;
+  int64_t count = 0;  // COMPACT: the kept count, once done
 };
 
 // While two or more batches run, admitted requests wait for the next launch
@@ -528,6 +532,8 @@ struct Slot {
   unsigned* hflag = nullptr;  // per request of the batch: 1 once its results are in memory; word kMaxBatch:
                               // 1 once the whole batch is done (pinned, mapped)
   unsigned* dflag = nullptr;  // the same flags' device address
+  int64_t* hcount = nullptr;  // per request: a compaction's kept count (pinned, mapped)
+  int64_t* dcount = nullptr;  // the same counts' device address
   bool busy = false;
   // Set once the batch's work and event are enqueued: until then the event
   // still describes the slot's previous batch (the launch may run on another
@@ -595,6 +601,7 @@ struct cox_server {
       e.ws = arena_mem + q.off + q.out_b;
       e.item0 = items;
       e.nitems = serve_items(q.r.n);
+      e.count = sl.dcount + i;
       items += e.nitems;
       compact = compact || q.r.kind == COX_REQ_COMPACT;
       q.state = kRunning;
@@ -602,7 +609,10 @@ struct cox_server {
     // (requests are < 2^31 elements each, so 2048 of them stay < 2^31 tiles)
     h->nitems = items;
     h->nreq = (int)ts.size();
-    for (size_t i = 0; i < ts.size(); ++i) __atomic_store_n(sl.hflag + i, 0u, __ATOMIC_RELAXED);
+    for (size_t i = 0; i < ts.size(); ++i) {
+      __atomic_store_n(sl.hflag + i, 0u, __ATOMIC_RELAXED);
+      sl.hcount[i] = 0;
+    }
     __atomic_store_n(sl.hflag + kMaxBatch, 0u, __ATOMIC_RELAXED);
     sl.t_checked = 0.0;
     sl.tickets = ts;
@@ -631,8 +641,8 @@ struct cox_server {
         c = cox_tile_scan(COX_SUM, (cox_dtype)d.dt, d.width, 256, d.in, d.out, d.n, d.flags, solo_st);
       } else if (d.kind == COX_REQ_COMPACT) {
         const size_t wsb = cox_ballot_compact_workspace(d.n, 256);
-        c = cox_ballot_compact((cox_dtype)d.dt, 32, 256, d.in, d.n, d.threshold, d.out,
-                               reinterpret_cast<int64_t*>(d.ws), d.ws + kAlign, wsb, 0u, solo_st);
+        c = cox_ballot_compact((cox_dtype)d.dt, 32, 256, d.in, d.n, d.threshold, d.out, d.count, d.ws + kAlign,
+                               wsb, 0u, solo_st);
       }
       if (d.kind == COX_REQ_REDUCE) {
         const unsigned nblk = (unsigned)d.nitems;
@@ -677,6 +687,7 @@ struct cox_server {
     if (it == reqs.end()) return;
     it->second.state = state;
     it->second.t_done = t;
+    if (state == kDone && it->second.r.kind == COX_REQ_COMPACT) it->second.count = sl.hcount[i];
     if (collect_finished) {
       finished.emplace_back(sl.tickets[i], t);
       nfinished.fetch_add(1, std::memory_order_release);
@@ -833,7 +844,9 @@ extern "C" cox_status cox_server_create(size_t budget_bytes, int max_requests, c
         cudaMallocHost(&sl.host_tab, tab) != cudaSuccess || cudaMalloc(&sl.dev_tab, tab) != cudaSuccess ||
         cudaMalloc(&sl.ctr, sizeof(SlotCtr)) != cudaSuccess || cudaMemset(sl.ctr, 0, sizeof(SlotCtr)) != cudaSuccess ||
         cudaHostAlloc(&sl.hflag, (kMaxBatch + 1) * sizeof(unsigned), cudaHostAllocMapped) != cudaSuccess ||
-        cudaHostGetDevicePointer((void**)&sl.dflag, sl.hflag, 0) != cudaSuccess) {
+        cudaHostGetDevicePointer((void**)&sl.dflag, sl.hflag, 0) != cudaSuccess ||
+        cudaHostAlloc(&sl.hcount, kMaxBatch * sizeof(int64_t), cudaHostAllocMapped) != cudaSuccess ||
+        cudaHostGetDevicePointer((void**)&sl.dcount, sl.hcount, 0) != cudaSuccess) {
       cox_server_destroy(s);
       return COX_ECUDA;
     }
@@ -949,22 +962,30 @@ extern "C" cox_status cox_server_wait(cox_server* s, uint64_t ticket, double tim
 
 extern "C" cox_status cox_server_result(cox_server* s, uint64_t ticket, void** d_out, int64_t* count) {
   if (!s || !d_out || !count) return COX_EINVAL;
-  cox_request r;
-  uint8_t* out;
-  size_t out_b;
+  std::lock_guard<std::mutex> g(s->mu);
+  auto it = s->reqs.find(ticket);
+  if (it == s->reqs.end() || it->second.state != kDone) return COX_EINVAL;
+  const cox_request& r = it->second.r;
+  *d_out = s->arena_mem + it->second.off;
+  *count = r.kind == COX_REQ_REDUCE ? 1 : r.kind == COX_REQ_SCAN ? r.n : it->second.count;
+  return COX_OK;
+}
+
+extern "C" cox_status cox_server_read(cox_server* s, uint64_t ticket, void* d_dst, int64_t words, void* stream) {
+  if (!s || words < 0 || (words > 0 && !d_dst)) return COX_EINVAL;
+  void* src;
+  int64_t count;
+  const cox_status c = cox_server_result(s, ticket, &src, &count);
+  if (c != COX_OK) return c;
   {
     std::lock_guard<std::mutex> g(s->mu);
     auto it = s->reqs.find(ticket);
-    if (it == s->reqs.end() || it->second.state != kDone) return COX_EINVAL;
-    r = it->second.r;
-    out = s->arena_mem + it->second.off;
-    out_b = it->second.out_b;
+    if (it == s->reqs.end() || (size_t)words * 4 > it->second.out_b) return COX_EINVAL;
   }
-  *d_out = out;
-  if (r.kind == COX_REQ_REDUCE) *count = 1;
-  else if (r.kind == COX_REQ_SCAN) *count = r.n;
-  else if (cudaMemcpy(count, out + out_b, sizeof(int64_t), cudaMemcpyDeviceToHost) != cudaSuccess) return COX_ECUDA;
-  return COX_OK;
+  if (words == 0) return COX_OK;
+  return cudaMemcpyAsync(d_dst, src, (size_t)words * 4, cudaMemcpyDeviceToDevice, as_stream(stream)) == cudaSuccess
+             ? COX_OK
+             : COX_ECUDA;
 }
 
 static void release_locked(cox_server* s, std::unordered_map<uint64_t, SReq>::iterator it) {
@@ -1021,6 +1042,7 @@ extern "C" void cox_server_destroy(cox_server* s) {
     if (sl.dev_tab) cudaFree(sl.dev_tab);
     if (sl.ctr) cudaFree(sl.ctr);
     if (sl.hflag) cudaFreeHost(sl.hflag);
+    if (sl.hcount) cudaFreeHost(sl.hcount);
   }
   if (s->arena_mem) cudaFree(s->arena_mem);
   delete s->arena;
