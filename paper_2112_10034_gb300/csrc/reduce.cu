@@ -98,14 +98,27 @@ __device__ __forceinline__ void copy_out_padded(const uint32_t* so, uint32_t* __
   for (int e = lane; e < cnt; e += 32) dst[e] = so[(e / NT) * P + (e % NT)];
 }
 
-// Persistent warps stream chunks of 32 rows through row_ring (load only);
+// Warps stream chunks of 32 rows through row_ring (load only);
 // lane t reduces row t's NT = 32 / W tiles in registers.  The chunk's
 // 32 x NT results (tiles (32c + t) NT + j, contiguous) are staged in the
 // chunk's own buffer -- free once every lane holds its row -- and leave by
 // coalesced warp stores; then the low words the same way.  The last n % 32 elements (a
 // partial row, padded) go to thread 0 of CTA 0.
+//
+// Plain reducers are bound by memory alone: one chunk per warp on one buffer,
+// CTAs handed out by the hardware, run 2^26 fp32 at W = 2 / 8 / 32 in 59.7 /
+// 45.9 / 42.0 us, against 65.2 / 47.2 / 43.9 as one persistent wave with three
+// buffers.  Compensated ones keep the wave: their arithmetic is longer than a
+// load, and their low words leave in a second pass over the buffer (W = 32
+// 45.0 us in either form; the block sums of reduce_block_rows.cuh lost: 43.4
+// against 47.6).
+template <class R>
+constexpr int tile_stages() {
+  return R::kComp ? kRedStages : 1;
+}
+
 template <class R, int W>
-__global__ void __launch_bounds__(kRingWarps * 32, 2)
+__global__ void __launch_bounds__(kRingWarps * 32, R::kComp ? 2 : 4)
     k_reduce_tile_rows(const __grid_constant__ CUtensorMap tin, const uint32_t* __restrict__ in,
                        uint32_t* __restrict__ out, float* __restrict__ lo, int64_t n, uint32_t limit,
                        unsigned* status) {
@@ -115,7 +128,8 @@ __global__ void __launch_bounds__(kRingWarps * 32, 2)
   const int lane = threadIdx.x & 31;
   const int64_t rows = n / 32;
   const int64_t ntiles = (n + W - 1) / W;
-  row_ring<false, kRedStages>(&tin, nullptr, rows, (rows + 31) / 32, 32, limit, status, [&](int64_t c, uint4* buf) {
+  row_ring<false, tile_stages<R>()>(&tin, nullptr, rows, (rows + 31) / 32, 32, limit, status,
+                                    [&](int64_t c, uint4* buf) {
     V v[32];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
@@ -372,15 +386,18 @@ static cox_status launch_reduce(cox_scope scope, const void* d_in, void* d_out, 
     CUtensorMap tin;
     if (!encode_rows32_map(&tin, d_in, rows, 32)) return COX_ECUDA;
     auto k = k_reduce_tile_rows<R, W>;
-    static int gmax_rows;
+    constexpr size_t smem_rows = ring_smem(tile_stages<R>());
+    static int grids[kMaxDevices];  // per device: the resident CTAs
+    int& gmax_rows = grids[device_index()];
     if (gmax_rows == 0) {
-      if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring_smem(kRedStages)) != cudaSuccess)
+      if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_rows) != cudaSuccess)
         return COX_ECUDA;
-      gmax_rows = persistent_grid(k, kRingWarps * 32, ring_smem(kRedStages), 1 << 30);
+      gmax_rows = persistent_grid(k, kRingWarps * 32, smem_rows, 1 << 30);
     }
-    const int64_t ctas = ((rows + 31) / 32 + kRingWarps - 1) / kRingWarps;
-    k<<<(int)(ctas < gmax_rows ? ctas : gmax_rows), kRingWarps * 32, ring_smem(kRedStages), st>>>(
-        tin, in, out, d_lo, n, spin_limit(), device_status_word());
+    const int64_t nch = (rows + 31) / 32;
+    unsigned ctas = ring_grid(nch, 1);
+    if (R::kComp && ctas > (unsigned)gmax_rows) ctas = (unsigned)gmax_rows;
+    k<<<ctas, kRingWarps * 32, smem_rows, st>>>(tin, in, out, d_lo, n, spin_limit(), device_status_word());
     return launch_status();
   }
   if (scope == COX_SCOPE_TILE) {
