@@ -306,9 +306,9 @@ size_t cox_integral_image_workspace(int64_t batch, int64_t height, int64_t width
  * cox_ballot_compact -- stable stream compaction driven by warp ballots.
  *
  * The filter of the SDK's filter_arr (Table 1) with a static, full-warp group:
- * b = ballot(key < threshold); rank = popc(b & lanes below); per-block scan of
- * warp counts; blocks ordered by a single-pass look-back over tile
- * descriptors.
+ * b = ballot(key < threshold); rank = popc(b & lanes below); per-tile scan of
+ * warp counts; tiles placed by the counts of all earlier tiles, published in
+ * per-tile descriptors.
  *   dt: COX_I32 (signed compare) or COX_U32 (unsigned compare).
  *   d_out: room for n elements; receives the kept keys in input order.
  *   d_count: one int64 on the device, receives the number kept.

@@ -293,8 +293,8 @@ extern "C" cox_status cox_ballot_compact(cox_dtype dt, int width, int block_dim,
 
 // ---------------------------------------------------------------------------
 // cox_ballot_compact_static: the same compaction for callers that cannot
-// allocate device memory.  Its scratch (the per-tile and per-group
-// look-back descriptors) lives in the fixed array below instead of a
+// allocate device memory.  Its scratch (the ticket and
+// the per-tile descriptors) lives in the fixed array below instead of a
 // caller-provided workspace.
 //
 // The array belongs to the library image: every GPU that loads libcox.so

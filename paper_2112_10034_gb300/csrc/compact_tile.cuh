@@ -1,16 +1,18 @@
-// Tile body of the ballot-driven stable compaction, shared by
-// cox_ballot_compact and the request server.
+// Tile body of the ballot-driven stable compaction (shared by
+// cox_ballot_compact, the aggregated filter and the request server), and the
+// request server's tile chaining.
 //
 // The filter of the SDK kernel filter_arr (Table 1 of the paper) with a
 // static, full-warp group instead of the dynamically coalesced one (the paper
 // covers non-divergent warp functions only, Section 2.2.3):
 //   b = __ballot_sync(full, key < t); rank = popc(b & lanemask_lt);
-// a shared-memory scan orders the warps of a tile, and tiles are ordered by a
-// single-pass decoupled look-back over per-tile descriptors.  A tile only
-// waits on tiles with smaller indexes, which callers hand out in order to
-// CTAs that already run, so the waits end; each wait is still bounded.
-// The look-back has two levels: within a group of 32 tiles, then over whole
-// groups (their counts summed by atomics as the last tile of each arrives).
+// a shared-memory scan orders the warps of a tile, and the counts of earlier
+// tiles place it.  A server batch holds the tiles of many requests, so there
+// each tile does its own decoupled look-back over per-tile descriptors: it only
+// waits on tiles with smaller indexes, which are handed out in order to CTAs
+// that already run, so the waits end; each wait is still bounded.  It has two
+// levels: within a group of 32 tiles, then over whole groups (their counts
+// summed by atomics as the last tile of each arrives).
 //
 // Tile layout: a tile of NW * 2048 keys sits in shared memory; warp w owns
 // the region of keys [2048w, 2048w + 2048) and compacts it in place to the
@@ -171,28 +173,6 @@ __device__ __forceinline__ int64_t look_back(uint64_t* desc, int64_t tile, int64
 // copies its kept keys to out[prefix + the warps before it ..]; the last
 // tile writes *d_count.
 constexpr int64_t kBigTile = 16384;  // elements per tile of the request server (64 KB)
-
-// key < thr as one 32-bit compare: thr is clamped into the key range first
-// (every key passes if thr is above the range, none if at or below it).
-struct KeepRule {
-  uint32_t t;  // keep iff key < t in the key's own signedness...
-  int mode;    // ...when mode == 0; mode 1 keeps all, mode 2 keeps none
-};
-
-template <bool SIGNED>
-__host__ __device__ inline KeepRule keep_rule(int64_t thr) {
-  const int64_t lo = SIGNED ? -(int64_t(1) << 31) : 0;
-  const int64_t hi = SIGNED ? (int64_t(1) << 31) - 1 : (int64_t(1) << 32) - 1;
-  if (thr > hi) return {0u, 1};
-  if (thr <= lo) return {0u, 2};
-  return {(uint32_t)thr, 0};
-}
-
-template <bool SIGNED>
-__device__ __forceinline__ bool keep_key(uint32_t k, KeepRule r) {
-  const bool lt = SIGNED ? (int32_t)k < (int32_t)r.t : k < r.t;
-  return r.mode == 0 ? lt : r.mode == 1;
-}
 
 // key < thr as one compare, key <= tm, in the key's own signedness: tm =
 // thr - 1 clamped into the key range; `none` when thr is at or below the

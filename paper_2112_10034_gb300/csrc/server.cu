@@ -25,7 +25,8 @@
 //           folds all partials in tile order;
 //   SCAN    every warp scans its 64 rows of 32 in place (shfl_up at the
 //           request's tile width) and the tile leaves by one TMA bulk store;
-//   COMPACT the big-tile compaction shared with cox_ballot_compact.
+//   COMPACT every warp compacts its 2048 keys (the body shared with
+//           cox_ballot_compact), a look-back places the tile.
 // A request's arithmetic depends only on the request, never on its batch.
 #include <algorithm>
 #include <atomic>

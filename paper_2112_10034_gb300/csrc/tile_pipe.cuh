@@ -126,6 +126,7 @@ __device__ __forceinline__ void tile_pipe(PipeShared<NB>& ps, Op& op, int nb, in
     PipePos at, ahead;  // the next tile; the one `flight` before it
     bool ok = true;
     int64_t k = 0;
+    int marked = 0;  // slots that have been told of the end
     unsigned t = 0;
     for (;; ++k) {
       if (k >= nb) ok = pipe_wait(ps, ps.free + at.slot, at.parity() ^ 1u, limit);
@@ -148,7 +149,10 @@ __device__ __forceinline__ void tile_pipe(PipeShared<NB>& ps, Op& op, int nb, in
         else mbar_arrive(ps.full + at.slot);
       }
       __syncwarp();
-      if (!more) break;
+      if (!more) {
+        marked = 1;
+        break;
+      }
       at.next(nb);
     }
     for (int i = 1; ok && i < ng; ++i) {  // the other groups hear of the end on the slots after
@@ -158,11 +162,11 @@ __device__ __forceinline__ void tile_pipe(PipeShared<NB>& ps, Op& op, int nb, in
         ps.tile[at.slot] = -1;
         mbar_arrive(ps.full + at.slot);
       }
+      marked += ok;
     }
-    if (ok) return;
-    give_up();
-    if (lane == 0)  // copies in flight land before the CTA ends
-      for (int64_t i = k > nb ? k - nb : 0; i < k; ++i)
+    if (!ok) give_up();
+    if (lane == 0)  // whatever becomes of the CTA, its copies in flight land before it ends
+      for (int64_t i = k + marked > nb ? k + marked - nb : 0; i < k; ++i)
         mbar_wait_bounded(ps.full + (int)(i % nb), (uint32_t)((i / nb) & 1), limit);
     __syncwarp();
     return;
