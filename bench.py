@@ -44,12 +44,12 @@ WORKLOAD = ("tile inclusive scan (shfl_up, cg tiles) of 2^26 fp32 N(0,1) at widt
 
 # DRAM bytes per launch of the dominant kernel from one ncu capture, valid
 # only while the kernel sources hash to `src_sha` (else reported as null).
-NCU_TRAFFIC = {"src_sha": "dc84082847ff3dcc",
+NCU_TRAFFIC = {"src_sha": "fbe74be0d7a526f4",
                "bytes_per_launch": {
-                                    "k_tile_scan_rows<Plain<AddF>, 16>": 268503296 + 216764416,
-                                    "k_tile_scan_rows<Comp, 16>": 268482816 + 216979456,
-                                    "k_tile_scan_rows<Plain<AddF>, 32>": 268469248 + 217031168,
-                                    "k_tile_scan_rows<Comp, 32>": 268507904 + 218467328}}
+                                    "k_tile_scan_rows<Plain<AddF>, 16>": 268454912 + 214578688,
+                                    "k_tile_scan_rows<Comp, 16>": 268472064 + 215199744,
+                                    "k_tile_scan_rows<Plain<AddF>, 32>": 268458240 + 213162752,
+                                    "k_tile_scan_rows<Comp, 32>": 268480000 + 215103488}}
 KERNEL_SOURCES = ["paper_2112_10034_gb300/csrc/scan.cu", "paper_2112_10034_gb300/csrc/cox_common.cuh"]
 
 
@@ -860,7 +860,8 @@ def run_profile(args):
     at density 0.5; `hist` runs 2^26-key Zipf match histograms; `batch` runs
     the batched kernel on 1000 arrays of the batched length law (~1e8
     elements); `gridscan` a 2^26 int32 grid-scope scan (`gridscan_comp`: fp32
-    compensated); `reduce` a 2^26 fp32
+    compensated); `blockscan` a 2^26 fp32 block-scope
+    scan at B 256, plain then compensated; `reduce` a 2^26 fp32
     compensated tile reduce (W 32) then block reduce (B 256); `intimage` the
     integral images of 64 8-bit 1080x1920 frames (a memset of the strip
     totals, then the strip walk), `intimage32` the same with 32-bit pixels; `filter` the
@@ -903,6 +904,14 @@ def run_profile(args):
         for _ in range(reps):
             chk(cox.cox_scan(0, 0, 2, 256, xi.data_ptr(), yi.data_ptr(), N_ELEMS, 0, 0, ws.data_ptr(), wsb, sh))
         launches = reps
+    elif args.profile == "blockscan":
+        xf = torch.from_numpy(inputs.normal_f32(N_ELEMS, inputs.BASE_SEED + 1)).to(dev)
+        yf = torch.empty_like(xf)
+        for _ in range(reps):
+            for comp in (False, True):
+                chk(cox.cox_scan(0, 2, 1, BLOCK, xf.data_ptr(), yf.data_ptr(), N_ELEMS,
+                                 cox.COX_F_COMPENSATED if comp else 0, 0, None, 0, sh))
+        launches = reps * 2
     elif args.profile == "gridscan_comp":
         xf = torch.from_numpy(inputs.normal_f32(N_ELEMS, inputs.BASE_SEED + 1)).to(dev)
         yf = torch.empty_like(xf)
@@ -975,7 +984,7 @@ def main():
     ap.add_argument("--no-secondary", action="store_true")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--cpu-seconds", type=float, default=12.0)
-    ap.add_argument("--profile", choices=["scan", "compact", "hist", "batch", "gridscan", "gridscan_comp", "reduce",
+    ap.add_argument("--profile", choices=["scan", "compact", "hist", "batch", "gridscan", "gridscan_comp", "blockscan", "reduce",
                                           "intimage", "intimage32", "filter", "coalesced"],
                     default=None,
                     help="small single-op case for ncu captures")

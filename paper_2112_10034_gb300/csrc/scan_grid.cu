@@ -900,7 +900,7 @@ using namespace cox;
 
 extern "C" size_t cox_scan_workspace(cox_scope scope, int64_t n) {
   if (scope != COX_SCOPE_GRID || n <= 0) return 0;
-  const int64_t t = (n + 8191) / 8192;  // enough for either tile size, plus group words
+  const int64_t t = (n + 8191) / 8192;  // enough for every form and tile size
   return scan_ws_bytes(t) + 24 * (size_t)((t + 31) / 32);
 }
 
