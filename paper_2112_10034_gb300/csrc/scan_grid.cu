@@ -142,30 +142,42 @@ __device__ typename R::V look_back_op(uint32_t* flags, uint64_t* agg, uint64_t* 
   return prefix;
 }
 
-// Published tile aggregates of the row-tile kernel, zero until written.  A
+// Published tile aggregates of the row-tile kernels, zero until written.  A
 // 32-bit value is one 64-bit word, (1 << 32) | bits; a compensated pair two,
 // one per 32-bit half, each with its own flag, so that every word read is
-// whole whatever order the halves arrive in.
-template <class R>
+// whole whatever order the halves arrive in.  PK: a pair in one word -- a flag
+// in bit 62, the error word rounded to 21 mantissa bits (about 2^-46 of the
+// sum) above the sum word -- for workspaces smaller than cox_scan_workspace().
+template <class R, bool PK>
 __host__ __device__ constexpr int agg_words() {
-  return R::kComp ? 2 : 1;
+  return R::kComp && !PK ? 2 : 1;
 }
-template <class R>
+template <class R, bool PK>
 __device__ __forceinline__ void agg_store(uint64_t* agg, int64_t tile, typename R::V v) {
-  if constexpr (R::kComp)
+  if constexpr (R::kComp && PK)
+    // (a carry of the rounding into the exponent is the next binade's value)
+    st_relaxed_u64(agg + tile, (1ull << 62) | ((((uint64_t)__float_as_uint(v.e) + 2u) >> 2 & 0x3FFFFFFFull) << 32) |
+                                   __float_as_uint(v.s));
+  else if constexpr (R::kComp)
     asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(agg + 2 * tile),
                  "l"((1ull << 32) | __float_as_uint(v.s)), "l"((1ull << 32) | __float_as_uint(v.e))
                  : "memory");
   else
     st_relaxed_u64(agg + tile, (1ull << 32) | to_bits(v));
 }
-// Whether the aggregate is there; its value.
-template <class R>
+// The aggregate as two flagged halves (a 32-bit value twice), zero flags while
+// it is not there.
+template <class R, bool PK>
 __device__ __forceinline__ void agg_load(const uint64_t* agg, int64_t tile, uint64_t (&w)[2]) {
-  if constexpr (R::kComp)
+  if constexpr (R::kComp && PK) {
+    const uint64_t q = ld_relaxed_u64(agg + tile), flag = (q >> 62) << 32;
+    w[0] = flag | (uint32_t)q;
+    w[1] = flag | (uint32_t)((uint32_t)(q >> 32) << 2);
+  } else if constexpr (R::kComp) {
     asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(w[0]), "=l"(w[1]) : "l"(agg + 2 * tile) : "memory");
-  else
+  } else {
     w[0] = w[1] = ld_relaxed_u64(agg + tile);
+  }
 }
 template <class R>
 __device__ __forceinline__ typename R::V agg_value(const uint64_t (&w)[2]) {
@@ -194,7 +206,7 @@ struct GridCfg {
 // A walk over the published aggregates in tile order (a whole warp): advances
 // from `cur` to `tile`, folding what it passes into `run`.  False if the
 // words did not appear within `limit` polls or `abort` was raised.
-template <class R>
+template <class R, bool PK>
 __device__ bool follow(const uint64_t* agg, int64_t tile, int64_t& cur, typename R::V& run, uint32_t limit,
                        volatile int* abort) {
   using V = typename R::V;
@@ -207,7 +219,7 @@ __device__ bool follow(const uint64_t* agg, int64_t tile, int64_t& cur, typename
     for (int v = 0; v < kWin; ++v) {
       const int64_t t = cur + v * 32 + lane;
       w[v][0] = w[v][1] = 0;
-      if (t < tile) agg_load<R>(agg, t, w[v]);
+      if (t < tile) agg_load<R, PK>(agg, t, w[v]);
     }
     V part = R::ident();
     int64_t step = 0;
@@ -398,7 +410,7 @@ constexpr size_t grid_scan_smem(int nb) {
   return 1024 + (size_t)nb * C::kTileBytes + sizeof(GridScanShared<R, C>);
 }
 
-template <class R, class C>
+template <class R, class C, bool PK>
 struct GridScanOp {
   using T = typename R::T;
   using V = typename R::V;
@@ -470,11 +482,11 @@ struct GridScanOp {
         sh->wtot[slot][k] = total;
         total = R::op(total, t);
       }
-      agg_store<R>(agg, tile, total);
+      agg_store<R, PK>(agg, tile, total);
     }
   }
   __device__ bool prefix(int slot, int64_t tile, uint32_t limit, volatile int* abort) {
-    if (!follow<R>(agg, tile, cur, run, limit, abort)) return false;
+    if (!follow<R, PK>(agg, tile, cur, run, limit, abort)) return false;
     if (lane_id() == 0) sh->prefix[slot] = run;
     return true;
   }
@@ -514,7 +526,7 @@ struct GridScanOp {
   }
 };
 
-template <class R>
+template <class R, bool PK>
 __global__ void __launch_bounds__(GridCfg<R>::kThreads, 1)
     k_scan_grid_rows(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtensorMap tout,
                      const uint32_t* __restrict__ in, uint32_t* __restrict__ out, int64_t n, unsigned* ticket,
@@ -524,7 +536,7 @@ __global__ void __launch_bounds__(GridCfg<R>::kThreads, 1)
   extern __shared__ uint8_t gsr_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(gsr_raw) + 1023) & ~uintptr_t(1023));
   GridScanShared<R, C>* sh = reinterpret_cast<GridScanShared<R, C>*>(base + (size_t)nb * C::kTileBytes);
-  GridScanOp<R, C> op{&tin, &tout, in, out, n, n / 32, agg, excl, reinterpret_cast<uint4*>(base), sh, 0,
+  GridScanOp<R, C, PK> op{&tin, &tout, in, out, n, n / 32, agg, excl, reinterpret_cast<uint4*>(base), sh, 0,
                    R::ident()};
   tile_pipe<C::kNB, C::kNW, 1>(sh->pipe, op, nb, flight, ntiles, ticket, limit, status);
 }
@@ -539,7 +551,7 @@ struct GridShortCfg {
   static constexpr uint32_t kTileBytes = kRows * 128;
 };
 
-template <class R>
+template <class R, bool PK>
 __global__ void __launch_bounds__(GridShortCfg::kNW * 32)
     k_scan_grid_short(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtensorMap tout,
                       const uint32_t* __restrict__ in, uint32_t* __restrict__ out, int64_t n, unsigned* ticket,
@@ -552,7 +564,7 @@ __global__ void __launch_bounds__(GridShortCfg::kNW * 32)
   __shared__ int64_t s_tile;
   __shared__ V s_part[C::kNW];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  GridScanOp<R, C> op{&tin, &tout, in, out, n, n / 32, agg, excl, reinterpret_cast<uint4*>(base), sh, 0,
+  GridScanOp<R, C, PK> op{&tin, &tout, in, out, n, n / 32, agg, excl, reinterpret_cast<uint4*>(base), sh, 0,
                       R::ident()};
   if (tid == 0) {
     mbar_init(sh->pipe.full, 1);
@@ -578,7 +590,7 @@ __global__ void __launch_bounds__(GridShortCfg::kNW * 32)
   for (int64_t t = tid; t < tile; t += C::kNW * 32) {
     uint64_t w[2];
     for (uint32_t polls = 0;; ++polls) {
-      agg_load<R>(agg, t, w);
+      agg_load<R, PK>(agg, t, w);
       if ((w[0] >> 32) != 0 && (w[1] >> 32) != 0) break;
       if (polls > limit) {
         ok = false;
@@ -817,6 +829,52 @@ inline ScanWs scan_ws(void* ws, int64_t ntiles) {
   return w;
 }
 
+// GRID scope over an aligned array of at least one full row.
+template <class R, bool PK>
+static cox_status launch_grid_rows(const uint32_t* in, uint32_t* out, int64_t n, int excl, void* ws, cudaStream_t st) {
+  if (!aligned16(ws)) return COX_EINVAL;
+  // Little more than one resident wave of one-tile CTAs (six per SM), or the
+  // pipeline.  2^22 int32 16.9 us against 20.2, 2^23 25.6 against 29.0, 1.26 x
+  // 10^7 31.7 against 30.5, 2^24 37.7 against 35.9; the smallest arrays also
+  // start sooner (10^4: 7.4 against 8.6).
+  const int64_t short_tiles = (n + GridShortCfg::kRows * 32 - 1) / (GridShortCfg::kRows * 32);
+  const bool use_short = short_tiles <= (int64_t)8 * sm_count();
+  using C = GridCfg<R>;
+  const int rows = use_short ? GridShortCfg::kRows : C::kRows;
+  const int64_t ntiles = use_short ? short_tiles : (n + C::kRows * 32 - 1) / (C::kRows * 32);
+  CUtensorMap tin, tout;
+  if (!encode_rows32_map(&tin, in, n / 32, rows) || !encode_rows32_map(&tout, out, n / 32, rows))
+    return COX_ECUDA;
+  // the ticket, then a zero aggregate per tile (within cox_scan_workspace)
+  if (cudaMemsetAsync(ws, 0, kScanWsHeader + (size_t)ntiles * agg_words<R, PK>() * 8, st) != cudaSuccess)
+    return COX_ECUDA;
+  unsigned* ticket = static_cast<unsigned*>(ws);
+  uint64_t* agg = reinterpret_cast<uint64_t*>(static_cast<char*>(ws) + kScanWsHeader);
+  if (use_short) {
+    k_scan_grid_short<R, PK><<<(unsigned)ntiles, GridShortCfg::kNW * 32, grid_scan_smem<R, GridShortCfg>(1), st>>>(
+        tin, tout, in, out, n, ticket, agg, excl, spin_limit(), device_status_word());
+    return launch_status();
+  }
+  auto k = k_scan_grid_rows<R, PK>;
+  static int grid[kMaxDevices];  // resident CTAs, per device
+  int& g = grid[device_index()];
+  if (g == 0) {
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)grid_scan_smem<R, C>(C::kNB)) !=
+        cudaSuccess)
+      return COX_ECUDA;
+    g = persistent_grid(k, C::kThreads, grid_scan_smem<R, C>(C::kNB), 1 << 30);
+  }
+  // as many buffers as give every CTA work: an array's tiles spread over the
+  // CTAs instead of queueing in the first ones; one that fits the buffers is
+  // loaded all at once
+  const int64_t ctas = ntiles < g ? ntiles : g;
+  const int nb = (int)std::min<int64_t>(C::kNB, (ntiles + ctas - 1) / ctas);
+  const int flight = ntiles <= ctas * nb ? nb : C::kFlight;
+  k<<<(unsigned)ctas, C::kThreads, grid_scan_smem<R, C>(nb), st>>>(tin, tout, in, out, n, ticket, agg, ntiles, excl,
+                                                                   nb, flight, spin_limit(), device_status_word());
+  return launch_status();
+}
+
 template <class R>
 static cox_status launch_scan_scope(cox_scope scope, int block, const void* d_in, void* d_out, int64_t n, int excl,
                                     void* ws, size_t ws_bytes, cudaStream_t st) {
@@ -834,48 +892,16 @@ static cox_status launch_scan_scope(cox_scope scope, int block, const void* d_in
     return launch_status();
   }
   if (n >= 32 && n / 32 < (int64_t(1) << 31) && aligned16(d_in) && aligned16(d_out)) {
-    if (!ws || ws_bytes < cox_scan_workspace(COX_SCOPE_GRID, n)) return COX_ENOMEM;
-    if (!aligned16(ws)) return COX_EINVAL;
-    // Little more than one resident wave of one-tile CTAs (six per SM), or the
-    // pipeline.  2^22 int32 16.9 us against 20.2, 2^23 25.6 against 29.0, 1.26 x
-    // 10^7 31.7 against 30.5, 2^24 37.7 against 35.9; the smallest arrays also
-    // start sooner (10^4: 7.4 against 8.6).
-    const int64_t short_tiles = (n + GridShortCfg::kRows * 32 - 1) / (GridShortCfg::kRows * 32);
-    const bool use_short = short_tiles <= (int64_t)8 * sm_count();
-    using C = GridCfg<R>;
-    const int rows = use_short ? GridShortCfg::kRows : C::kRows;
-    const int64_t ntiles = use_short ? short_tiles : (n + C::kRows * 32 - 1) / (C::kRows * 32);
-    CUtensorMap tin, tout;
-    if (!encode_rows32_map(&tin, d_in, n / 32, rows) || !encode_rows32_map(&tout, d_out, n / 32, rows))
-      return COX_ECUDA;
-    // the ticket, then a zero aggregate per tile (within cox_scan_workspace)
-    if (cudaMemsetAsync(ws, 0, kScanWsHeader + (size_t)ntiles * agg_words<R>() * 8, st) != cudaSuccess)
-      return COX_ECUDA;
-    unsigned* ticket = static_cast<unsigned*>(ws);
-    uint64_t* agg = reinterpret_cast<uint64_t*>(static_cast<char*>(ws) + kScanWsHeader);
-    if (use_short) {
-      k_scan_grid_short<R><<<(unsigned)ntiles, GridShortCfg::kNW * 32, grid_scan_smem<R, GridShortCfg>(1), st>>>(
-          tin, tout, in, out, n, ticket, agg, excl, spin_limit(), device_status_word());
-      return launch_status();
+    const bool whole = ws_bytes >= cox_scan_workspace(COX_SCOPE_GRID, n);
+    if constexpr (R::kComp) {
+      // compensated sums also take the workspace of 16384-element tiles (about
+      // half of cox_scan_workspace()), with packed aggregates
+      const int64_t t = (n + 16383) / 16384;
+      if (ws && !whole && ws_bytes >= scan_ws_bytes(t) + 24 * (size_t)((t + 31) / 32))
+        return launch_grid_rows<R, true>(in, out, n, excl, ws, st);
     }
-    auto k = k_scan_grid_rows<R>;
-    static int grid[kMaxDevices];  // resident CTAs, per device
-    int& g = grid[device_index()];
-    if (g == 0) {
-      if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)grid_scan_smem<R, C>(C::kNB)) !=
-          cudaSuccess)
-        return COX_ECUDA;
-      g = persistent_grid(k, C::kThreads, grid_scan_smem<R, C>(C::kNB), 1 << 30);
-    }
-    // as many buffers as give every CTA work: an array's tiles spread over the
-    // CTAs instead of queueing in the first ones; one that fits the buffers is
-    // loaded all at once
-    const int64_t ctas = ntiles < g ? ntiles : g;
-    const int nb = (int)std::min<int64_t>(C::kNB, (ntiles + ctas - 1) / ctas);
-    const int flight = ntiles <= ctas * nb ? nb : C::kFlight;
-    k<<<(unsigned)ctas, C::kThreads, grid_scan_smem<R, C>(nb), st>>>(tin, tout, in, out, n, ticket, agg, ntiles, excl,
-                                                                     nb, flight, spin_limit(), device_status_word());
-    return launch_status();
+    if (!ws || !whole) return COX_ENOMEM;
+    return launch_grid_rows<R, false>(in, out, n, excl, ws, st);
   }
   constexpr int TILE = grid_scan_tile<R>();
   const int64_t ntiles = (n + TILE - 1) / TILE;

@@ -140,3 +140,27 @@ def test_compaction_forms_agree(cox, where, delta, d):  # noqa: F811
             assert int(cnt.item()) == want.numel() and torch.equal(out[:want.numel()], want)
             assert bool((out[n:] == POISON).all())
     assert cox.device_status() == cox.COX_OK
+
+
+@pytest.mark.parametrize("n", [32, 100_003, 3_000_001, 30_000_007])
+def test_compensated_grid_scan_takes_the_smaller_workspace(cox, n):  # noqa: F811
+    """Half of cox_scan_workspace(): aggregates packed into one word each."""
+    import torch
+    def align(b):
+        return (b + 255) // 256 * 256
+    t = -(-n // 16384)
+    need = 256 + align(4 * t) + 16 * t + 24 * (-(-t // 32))
+    x = torch.from_numpy(inputs.normal_f32(n, seed=n)).cuda()
+    ws = torch.full((max(need, cox.cox_scan_workspace(o.GRID, n)),), 0xA5, dtype=torch.uint8, device="cuda")
+    out = poisoned(n, torch.float32)
+
+    def call(bytes_, comp=1):
+        return cox.cox_scan(o.SUM, o.F32, o.GRID, 256, x.data_ptr(), out.data_ptr(), n, comp, 0, ws.data_ptr(), bytes_,
+                            None)
+    assert call(need - 1) == cox.COX_ENOMEM
+    assert call(cox.cox_scan_workspace(o.GRID, n) - 1, 0) == cox.COX_ENOMEM
+    assert call(need) == cox.COX_OK
+    want = x.double().cumsum(0)
+    err = (out[:n].double() - want).abs() / torch.maximum(want.abs(), 2.0**-24 * x.double().abs().cumsum(0))
+    assert float(err.max()) <= 1e-5
+    assert bool((ws[need:] == 0xA5).all())
