@@ -542,7 +542,6 @@ class Server:
 
     def __init__(self, budget_bytes: int, max_requests: int = 1024):
         self.handle = ctypes.c_void_p()
-        self._device = _torch().device("cuda", _torch().cuda.current_device())  # the server's
         _check(lib().cox_server_create(int(budget_bytes), int(max_requests), ctypes.byref(self.handle)),
                "cox_server_create")
         self._keep = {}
@@ -574,7 +573,7 @@ class Server:
         _check(lib().cox_server_wait(self.handle, ticket, float(timeout_s)), "cox_server_wait")
 
     def result(self, ticket: int, req: cox_request):
-        """A copy (torch CUDA tensor) of a done request's output."""
+        """A copy of a done request's output: a tensor on the current device, made on its current stream."""
         t = _torch()
         h = lib()
         if req.kind == COX_REQ_COMPACT:
@@ -584,8 +583,8 @@ class Server:
             n = c.value
         else:
             n = 2 if req.kind == COX_REQ_REDUCE else req.n
-        out = t.empty(n, dtype=t.float32 if req.dt == COX_F32 else t.int32, device=self._device)
-        _check(h.cox_server_read(self.handle, ticket, out.data_ptr(), n, _stream(self._device)), "cox_server_result")
+        out = t.empty(n, dtype=t.float32 if req.dt == COX_F32 else t.int32, device="cuda")
+        _check(h.cox_server_read(self.handle, ticket, out.data_ptr(), n, _stream(None)), "cox_server_result")
         return out
 
     def release(self, ticket: int) -> None:
