@@ -576,13 +576,12 @@ class Server:
         """A copy of a done request's output: a tensor on the current device, made on its current stream."""
         t = _torch()
         h = lib()
-        if req.kind == COX_REQ_COMPACT:
+        n = 2
+        if req.kind != COX_REQ_REDUCE:  # the server's count: `req` may have been filled anew since it was submitted
             p = ctypes.c_void_p()
             c = ctypes.c_int64()
             _check(h.cox_server_result(self.handle, ticket, ctypes.byref(p), ctypes.byref(c)), "cox_server_result")
             n = c.value
-        else:
-            n = 2 if req.kind == COX_REQ_REDUCE else req.n
         out = t.empty(n, dtype=t.float32 if req.dt == COX_F32 else t.int32, device="cuda")
         _check(h.cox_server_read(self.handle, ticket, out.data_ptr(), n, _stream(None)), "cox_server_result")
         return out

@@ -71,3 +71,15 @@ def test_the_copy_is_ordered_on_the_device_that_holds_it(kind, monkeypatch):
     srv.result(1, c.cox_request(kind, c.COX_I32, 32, 0, 7, 0, 16))
     assert [o[2] for o in torch.outs] == [1]
     assert torch.streams == [1]
+
+
+@pytest.mark.parametrize("kind", [c.COX_REQ_SCAN, c.COX_REQ_COMPACT])
+def test_the_length_is_the_servers(kind, monkeypatch):
+    """A program may fill one request structure anew for each submission: it no
+    longer describes the request whose result is read."""
+    torch, lib = FakeTorch(current=0), FakeLib(7)
+    srv = _server(monkeypatch, torch, lib)
+    req = c.cox_request(kind, c.COX_I32, 32, 0, 7, 0, 16)
+    req.n = 3
+    srv.result(1, req)
+    assert lib.words == [7] and torch.outs[0][0] == 7
