@@ -585,10 +585,13 @@ cox_status cox_server_result(cox_server* s, uint64_t ticket, void** d_out, int64
 /* Copies the first `words` 32-bit words of a done request's output to d_dst on
  * `stream` (REDUCE: 2, the element and its low word).  COX_EINVAL for a ticket
  * that is not done or more words than the output's room.  The request may be
- * released once the copy is done. */
+ * released as soon as the call returns: its memory is given back when the copy
+ * is done (not so for a copy into a graph that is being captured, which needs
+ * the request until it has run). */
 cox_status cox_server_read(cox_server* s, uint64_t ticket, void* d_dst, int64_t words, void* stream);
 
-/* Frees a done request's arena memory and slot. */
+/* Frees a done request's slot, and its arena memory once the copies that
+ * cox_server_read enqueued are done. */
 cox_status cox_server_release(cox_server* s, uint64_t ticket);
 
 cox_status cox_server_get_stats(cox_server* s, cox_server_stats* st);
