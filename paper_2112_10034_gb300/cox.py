@@ -582,8 +582,9 @@ class Server:
             c = ctypes.c_int64()
             _check(h.cox_server_result(self.handle, ticket, ctypes.byref(p), ctypes.byref(c)), "cox_server_result")
             n = c.value
-        out = t.empty(n, dtype=t.float32 if req.dt == COX_F32 else t.int32, device="cuda")
-        _check(h.cox_server_read(self.handle, ticket, out.data_ptr(), n, _stream(None)), "cox_server_result")
+        dev = t.cuda.current_device()
+        out = t.empty(n, dtype=t.float32 if req.dt == COX_F32 else t.int32, device=dev)
+        _check(h.cox_server_read(self.handle, ticket, out.data_ptr(), n, _stream(dev)), "cox_server_result")
         return out
 
     def release(self, ticket: int) -> None:

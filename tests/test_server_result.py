@@ -12,7 +12,7 @@ class FakeTorch:
     float32, int32 = "float32", "int32"
 
     def __init__(self, current):
-        self.cuda = types.SimpleNamespace(current_device=lambda: current, current_stream=self._stream)
+        self.cuda = types.SimpleNamespace(current_device=lambda: self.current, current_stream=self._stream)
         self.current = current
         self.outs, self.streams = [], []
 
