@@ -257,7 +257,10 @@ __device__ __forceinline__ void tile_pipe(PipeShared<NB>& ps, Op& op, int nb, in
     // for its fold).
     __nanosleep(20);
     if (__any_sync(kFull, ps.abort)) return;
-    if (++spin > limit) {
+    // A look at both takes 0.18 us, a poll of the other warps' waits up to 1 us:
+    // counted alike, the workers would end a CTA whose prefix warp has most of
+    // its polls left.
+    if ((++spin >> 4) > limit) {
       give_up();
       return;
     }
