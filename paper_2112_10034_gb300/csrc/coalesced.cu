@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(32 * kFilterWarps, 6)
     atomicOr(status, (unsigned)kDevTimeout);
     for (int64_t j = it; j < it + kFilterStages; ++j)  // iterations it .. it + stages - 1 were issued
       if (blockIdx.x + j * G < nfull)
-        mbar_wait_bounded(bar + (int)(j % kFilterStages), (uint32_t)((j / kFilterStages) & 1), limit);
+        mbar_drain(bar + (int)(j % kFilterStages), (uint32_t)((j / kFilterStages) & 1));
   }
 }
 

@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(kCompactThreads, 6)
   if (__syncthreads_or(!mbar_wait_bounded(sh->pipe.full, 0u, limit))) {
     if (tid == 0) {
       atomicOr(status, (unsigned)kDevTimeout);
-      mbar_wait_bounded(sh->pipe.full, 0u, limit);
+      mbar_drain(sh->pipe.full, 0u);
     }
     return;
   }

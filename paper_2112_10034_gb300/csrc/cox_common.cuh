@@ -547,6 +547,15 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
   return false;
 }
 
+// The wait for a copy in flight before its CTA ends, after another wait ran
+// out: bounded by itself (65 ms and more), since under a spin limit of a few
+// polls a copy may well land after them -- in shared memory that is by then
+// another CTA's.
+constexpr uint32_t kDrainPolls = 1u << 16;
+__device__ __forceinline__ void mbar_drain(uint64_t* bar, uint32_t parity) {
+  mbar_wait_bounded(bar, parity, kDrainPolls);
+}
+
 // --------------------------------------------------- per-warp row ring
 // Streams chunks of `rpc` rows x 32 elements (4 KB for 32 rows) of a tensor
 // map built by encode_rows32_map (box 32 x rpc) through a ring of NS buffers
@@ -631,7 +640,7 @@ __device__ __forceinline__ void row_ring(const CUtensorMap* tin, const CUtensorM
       atomicOr(status, 1u);  // kDevTimeout
       for (int j = 0; j < AHEAD; ++j) {
         const int64_t kk = k + j;
-        if (gw + kk * nw < nch) mbar_wait_bounded(bars + (int)(kk % NS), (uint32_t)((kk / NS) & 1), limit);
+        if (gw + kk * nw < nch) mbar_drain(bars + (int)(kk % NS), (uint32_t)((kk / NS) & 1));
       }
     }
     if constexpr (STORE) tma_store_wait_read();  // (the copies' writes are complete when the kernel is)

@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(kGbThreads) k_grid_bcast(const uint32_t* in, u
     if (!s_loaded) {
       if (tid == 0) {
         atomicOr(status, (unsigned)kDevTimeout);
-        mbar_wait_bounded(&s_bar, 0, limit);  // the copies in flight, before the CTA ends
+        mbar_drain(&s_bar, 0);  // the copies in flight, before the CTA ends
       }
     } else {
       for (int64_t i = tid; i < len; i += kGbThreads) acc.add(gb_smem[i]);

@@ -809,7 +809,7 @@ __global__ void __launch_bounds__(96 * StripCfg<DT>::NP, 1)
   if (!ok && lane == 0) {
     atomicOr(status, kDevTimeout);
     for (int64_t q = jw.q; q < ji.q; ++q)  // copies still in flight land before the warp exits
-      mbar_wait_bounded(full + (int)(q % NS), (uint32_t)((q / NS) & 1), limit);
+      mbar_drain(full + (int)(q % NS), (uint32_t)((q / NS) & 1));
   }
   __syncwarp();
 }

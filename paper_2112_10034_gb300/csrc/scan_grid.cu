@@ -285,7 +285,7 @@ __global__ void __launch_bounds__(256) k_scan_grid(const uint32_t* __restrict__ 
     if (__syncthreads_or(!ok)) {
       if (tid == 0) {
         atomicOr(status, (unsigned)kDevTimeout);
-        mbar_wait_bounded(bar, 0u, limit);
+        mbar_drain(bar, 0u);
         st_relaxed_u64(inc + tile, pack<R>(R::ident()));
         st_release_u32(flags + tile, 2u);
       }
@@ -578,7 +578,7 @@ __global__ void __launch_bounds__(GridShortCfg::kNW * 32)
   if (__syncthreads_or(!mbar_wait_bounded(sh->pipe.full, 0u, limit))) {
     if (tid == 0) {
       atomicOr(status, (unsigned)kDevTimeout);
-      mbar_wait_bounded(sh->pipe.full, 0u, limit);
+      mbar_drain(sh->pipe.full, 0u);
     }
     return;
   }

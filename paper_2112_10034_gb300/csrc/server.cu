@@ -319,7 +319,7 @@ __device__ __forceinline__ void serve_body(const ReqDesc* reqs, int nreq, int64_
       if (__syncthreads_or(!ok)) {
         if (tid == 0) {
           atomicOr(status, (unsigned)kDevTimeout);
-          mbar_wait_bounded(bar, (loads - 1) & 1u, limit);  // the copy in flight, before the CTA ends
+          mbar_drain(bar, (loads - 1) & 1u);  // the copy in flight, before the CTA ends
         }
         break;
       }

@@ -167,7 +167,7 @@ __device__ __forceinline__ void tile_pipe(PipeShared<NB>& ps, Op& op, int nb, in
     if (!ok) give_up();
     if (lane == 0)  // whatever becomes of the CTA, its copies in flight land before it ends
       for (int64_t i = k + marked > nb ? k + marked - nb : 0; i < k; ++i)
-        mbar_wait_bounded(ps.full + (int)(i % nb), (uint32_t)((i / nb) & 1), limit);
+        mbar_drain(ps.full + (int)(i % nb), (uint32_t)((i / nb) & 1));
     __syncwarp();
     return;
   }
