@@ -1,8 +1,8 @@
 // cox_ballot_compact: stable stream compaction from warp ballots.
 //
 // Tiles of 8192 keys (32 KB) arrive by TMA bulk copies (plain loads for a
-// ragged or unaligned tile) and go through the tile pipeline (tile_pipe.cuh;
-// short arrays: one tile per CTA).  In a tile, by eight warps:
+// ragged tile) and go through the tile pipeline (tile_pipe.cuh; short arrays:
+// one tile per CTA).  In a tile, by eight warps:
 //   fold    every warp compacts its 1024 keys in place in one pass
 //           (compact_tile.cuh): per chunk of 128 keys, b =
 //           __ballot_sync(keep) for each of a lane's four key slots, rank =
@@ -24,6 +24,15 @@ constexpr int kCompactNW = kCompactThreads / 32;
 constexpr int kCompactReg = 1024;                            // keys per warp
 constexpr int64_t kCompactTile = kCompactNW * kCompactReg;  // 8192 keys
 constexpr uint32_t kCompactTileBytes = (uint32_t)kCompactTile * 4;
+// Room of a tile in shared memory.  A bulk copy starts and ends on 16-byte
+// boundaries: an array that begins `shift` words past one is copied from the
+// boundary before the tile to the one after it (words of the neighbouring
+// tiles, never beyond the array) and its tile sits `shift` words into the
+// buffer.  The first tile, and one whose copy would pass the array's end, are
+// loaded word by word.  2^28 keys 4 bytes off, d = 0.1 / 0.5 / 0.9: 256 / 291 / 331 us;
+// loaded word by word in fold, which every later tile waits for, 703 / 751 /
+// 789 (577 / 649 / 715 by the cooperative kernel before the pipeline).
+constexpr int kCompactBuf = (int)kCompactTile + 4;
 // Shape of the pipeline, one CTA per SM: six tiles, two groups of eight worker
 // warps, three loads in flight.  2^28 keys at d = 0.1 / 0.5 / 0.9: 249 / 283 /
 // 323 us (4740 / 5700 / 6310 GB/s); one group 344 / 367 / 394, three 252 / 283
@@ -61,20 +70,23 @@ struct CompactOp {
   int64_t* d_count;
   uint64_t* desc;
   int64_t ntiles;
-  int vec;
+  int shift;  // words of `keys` past a 16-byte boundary
   uint32_t* bufs;
   CompactShared<NB>* sh;
   static constexpr int kWin = 8;  // 32-tile rows per poll of the walk
   int64_t cur = 0, run = 0, base = 0;  // the prefix warp's walk (as AggWalk of the grid scan)
 
-  __device__ uint32_t* buf(int slot) const { return bufs + (size_t)slot * kCompactTile; }
-  __device__ bool bulk(int64_t tile) const { return vec && (tile + 1) * kCompactTile <= n; }
+  __device__ uint32_t* buf(int slot) const { return bufs + (size_t)slot * kCompactBuf + shift; }
+  __device__ bool bulk(int64_t tile) const {
+    return shift == 0 ? (tile + 1) * kCompactTile <= n : tile > 0 && (tile + 1) * kCompactTile + 4 - shift <= n;
+  }
 
   __device__ void load(int slot, int64_t tile) const {
     uint64_t* bar = sh->pipe.full + slot;
     if (bulk(tile)) {
-      mbar_arrive_expect_tx(bar, kCompactTileBytes);
-      tma_load_1d(buf(slot), keys + tile * kCompactTile, kCompactTileBytes, bar);
+      const uint32_t bytes = kCompactTileBytes + (shift ? 16u : 0u);
+      mbar_arrive_expect_tx(bar, bytes);
+      tma_load_1d(buf(slot) - shift, keys + tile * kCompactTile - shift, bytes, bar);
     } else {
       mbar_arrive(bar);
     }
@@ -159,10 +171,10 @@ template <bool SIGNED>
 __global__ void __launch_bounds__(kCompactPipeThreads, 1)
     k_ballot_compact(const uint32_t* __restrict__ keys, int64_t n, int64_t thr, uint32_t* __restrict__ out,
                      int64_t* __restrict__ d_count, unsigned* ticket, uint64_t* desc, int64_t ntiles, int nb,
-                     int flight, uint32_t limit, unsigned* status, int vec) {
+                     int flight, uint32_t limit, unsigned* status, int shift) {
   extern __shared__ __align__(16) uint32_t smem[];
-  auto* sh = reinterpret_cast<CompactShared<kCompactNB>*>(smem + (size_t)nb * kCompactTile);
-  CompactOp<SIGNED, kCompactNB> op{keys, n, le_rule<SIGNED>(thr), out, d_count, desc, ntiles, vec, smem, sh};
+  auto* sh = reinterpret_cast<CompactShared<kCompactNB>*>(smem + (size_t)nb * kCompactBuf);
+  CompactOp<SIGNED, kCompactNB> op{keys, n, le_rule<SIGNED>(thr), out, d_count, desc, ntiles, shift, smem, sh};
   tile_pipe<kCompactNB, kCompactNW, kCompactNG>(sh->pipe, op, nb, flight, ntiles, ticket, limit, status);
 }
 
@@ -172,13 +184,13 @@ template <bool SIGNED>
 __global__ void __launch_bounds__(kCompactThreads, 6)
     k_ballot_compact_short(const uint32_t* __restrict__ keys, int64_t n, int64_t thr, uint32_t* __restrict__ out,
                            int64_t* __restrict__ d_count, unsigned* ticket, uint64_t* desc, int64_t ntiles,
-                           uint32_t limit, unsigned* status, int vec) {
+                           uint32_t limit, unsigned* status, int shift) {
   extern __shared__ __align__(16) uint32_t smem[];
-  auto* sh = reinterpret_cast<CompactShared<1>*>(smem + kCompactTile);
+  auto* sh = reinterpret_cast<CompactShared<1>*>(smem + kCompactBuf);
   __shared__ int64_t s_tile;
   __shared__ uint32_t s_part[kCompactNW];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  CompactOp<SIGNED, 1> op{keys, n, le_rule<SIGNED>(thr), out, d_count, desc, ntiles, vec, smem, sh};
+  CompactOp<SIGNED, 1> op{keys, n, le_rule<SIGNED>(thr), out, d_count, desc, ntiles, shift, smem, sh};
   if (tid == 0) {
     mbar_init(sh->pipe.full, 1);
     mbar_init_fence();
@@ -256,19 +268,19 @@ extern "C" cox_status cox_ballot_compact(cox_dtype dt, int width, int block_dim,
   const int64_t ntiles = (n + tile - 1) / tile;
   unsigned* ticket = static_cast<unsigned*>(d_workspace);  // in the header, zero like the descriptors
   uint64_t* desc = reinterpret_cast<uint64_t*>(static_cast<char*>(d_workspace) + kCompactWsHeader);
-  const int vec = aligned16(d_keys);
+  const int shift = (int)(reinterpret_cast<uintptr_t>(d_keys) % 16 / 4);
   const uint32_t* keys = static_cast<const uint32_t*>(d_keys);
   uint32_t* outp = static_cast<uint32_t*>(d_out);
   if (ntiles <= (int64_t)kCompactShortTiles * sm_count()) {
-    const size_t smem = kCompactTileBytes + sizeof(CompactShared<1>);
+    const size_t smem = kCompactBuf * 4 + sizeof(CompactShared<1>);
     auto go = [&](auto kern) {
       kern<<<(unsigned)ntiles, kCompactThreads, smem, st>>>(keys, n, threshold, outp, d_count, ticket, desc, ntiles,
-                                                            spin_limit(), device_status_word(), vec);
+                                                            spin_limit(), device_status_word(), shift);
       return launch_status();
     };
     return dt == COX_I32 ? go(k_ballot_compact_short<true>) : go(k_ballot_compact_short<false>);
   }
-  auto smem = [](int nb) { return (size_t)nb * kCompactTileBytes + sizeof(CompactShared<kCompactNB>); };
+  auto smem = [](int nb) { return (size_t)nb * kCompactBuf * 4 + sizeof(CompactShared<kCompactNB>); };
   auto launch = [&](auto kern, int* grid) {
     int& g = grid[device_index()];
     if (g == 0) {
@@ -284,7 +296,7 @@ extern "C" cox_status cox_ballot_compact(cox_dtype dt, int width, int block_dim,
     const int flight = ntiles <= ctas * nb ? nb : kCompactFlight;
     kern<<<(unsigned)ctas, kCompactPipeThreads, smem(nb), st>>>(keys, n, threshold, outp, d_count, ticket, desc,
                                                                 ntiles, nb, flight, spin_limit(),
-                                                                device_status_word(), vec);
+                                                                device_status_word(), shift);
     return launch_status();
   };
   static int grid_s[kMaxDevices], grid_u[kMaxDevices];  // resident CTAs, per device

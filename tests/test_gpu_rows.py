@@ -142,6 +142,27 @@ def test_compaction_forms_agree(cox, where, delta, d):  # noqa: F811
     assert cox.device_status() == cox.COX_OK
 
 
+@pytest.mark.parametrize("off", [1, 2, 3])
+@pytest.mark.parametrize("tiles", [1, 2, "pipe"])
+@pytest.mark.parametrize("delta", [-1, 0, 1, 2, 3, 4])
+def test_compaction_of_unaligned_arrays(cox, off, tiles, delta):  # noqa: F811
+    """Tiles copied from the 16-byte boundary before them; the ends of the array."""
+    import torch
+    t = 7 * torch.cuda.get_device_properties(0).multi_processor_count if tiles == "pipe" else tiles
+    n = t * 8192 + delta
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n)
+    keys = torch.randint(-2**31, 2**31 - 1, (n + off,), generator=g, device="cuda", dtype=torch.int32)[off:]
+    assert keys.data_ptr() % 16 == 4 * off
+    for where in ("apart", "in place"):
+        want = keys[keys < 0]
+        out = poisoned(n, torch.int32) if where == "apart" else keys
+        _, cnt = cox.ballot_compact(keys, 0, out=out)
+        assert int(cnt.item()) == want.numel() and torch.equal(out[:want.numel()], want)
+        assert where == "in place" or bool((out[want.numel():] == POISON).all())
+    assert cox.device_status() == cox.COX_OK
+
+
 @pytest.mark.parametrize("n", [32, 100_003, 3_000_001, 30_000_007])
 def test_compensated_grid_scan_takes_the_smaller_workspace(cox, n):  # noqa: F811
     """Half of cox_scan_workspace(): aggregates packed into one word each."""
