@@ -185,6 +185,97 @@ __device__ __forceinline__ typename R::V agg_value(const uint64_t (&w)[2]) {
   else return from_bits<typename R::T>((uint32_t)w[0]);
 }
 
+// Look-back of the short form's 32-bit sums (wrapping adds, so that a group's
+// sum can be taken by atomics in any order): desc[t] = (state << 32) | value,
+// state 0 nothing, 1 aggregate, 2 inclusive prefix.  Tiles form groups of 32;
+// a tile adds (1 << 48) | value to its group's accumulator gacc[g] after
+// publishing its aggregate, and the add that completes the group publishes the
+// group aggregate in gdesc[g]; the last tile of a group also puts its
+// inclusive prefix there (atomicMax: a state-2 word is larger than any state-1
+// word).  The look-back reads the tile's own group first, then whole groups,
+// 32 per window (1024 tiles): a few lines, where reading every earlier
+// aggregate has all CTAs poll all lines while they are being written.  Called
+// by a whole warp; a wait that runs out publishes a zero prefix.
+__device__ unsigned look_back_sum2(uint64_t* desc, uint64_t* gdesc, uint64_t* gacc, int64_t tile, int64_t ntiles,
+                                   unsigned total, uint32_t limit, unsigned* status, bool& gave_up) {
+  const int lane = lane_id();
+  gave_up = false;
+  const int64_t g = tile >> 5;
+  const int pos = (int)(tile & 31);
+  if (lane == 0) {
+    st_relaxed_u64(desc + tile, ((tile == 0 ? 2ull : 1ull) << 32) | total);
+    const int64_t gsize = min((int64_t)32, ntiles - (g << 5));
+    const unsigned long long old = atomicAdd(reinterpret_cast<unsigned long long*>(gacc + g), (1ull << 48) | total);
+    if ((int64_t)(old >> 48) + 1 == gsize)
+      atomicMax(reinterpret_cast<unsigned long long*>(gdesc + g), (1ull << 32) | (uint32_t)(old + total));
+  }
+  unsigned prefix = 0;
+  uint32_t polls = 0;
+  bool timed_out = false;
+  bool done = tile == 0;
+  if (!done && pos > 0) {  // own group: lane l holds position l < pos
+    const int64_t g0 = g << 5;
+    uint64_t d = lane < pos ? ld_relaxed_u64(desc + g0 + lane) : (1ull << 32);
+    unsigned pm;
+    int fl;
+    for (;;) {
+      pm = __ballot_sync(kFull, lane < pos && (d >> 32) == 2u);
+      fl = pm ? 31 - __clz(pm) : -1;
+      const bool missing = lane < pos && lane > fl && (d >> 32) == 0u;
+      if (!__any_sync(kFull, missing)) break;
+      if (++polls > limit) {
+        timed_out = true;
+        break;
+      }
+      if (polls > 64) __nanosleep(64);
+      if (missing) d = ld_relaxed_u64(desc + g0 + lane);
+    }
+    if (!__any_sync(kFull, timed_out)) {
+      unsigned v = (lane < pos && lane >= fl) ? (unsigned)d : 0u;
+      prefix = __reduce_add_sync(kFull, v);
+      done = fl >= 0;
+    }
+  }
+  if (!done && !__any_sync(kFull, timed_out)) {  // whole groups: lane l holds group gw - l
+    for (int64_t gw = g - 1;; gw -= 32) {
+      const int64_t gi = gw - lane;
+      uint64_t d = gi >= 0 ? ld_relaxed_u64(gdesc + gi) : (2ull << 32);  // before group 0: 0
+      unsigned pm;
+      for (;;) {
+        pm = __ballot_sync(kFull, (d >> 32) == 2u);
+        const int fl = pm ? __ffs(pm) - 1 : 32;
+        const bool missing = lane <= fl && (d >> 32) == 0u;
+        if (!__any_sync(kFull, missing)) break;
+        if (++polls > limit) {
+          timed_out = true;
+          break;
+        }
+        if (polls > 64) __nanosleep(64);
+        if (missing && gi >= 0) d = ld_relaxed_u64(gdesc + gi);
+      }
+      if (__any_sync(kFull, timed_out)) break;
+      const int fl = pm ? __ffs(pm) - 1 : 32;
+      prefix += __reduce_add_sync(kFull, lane <= fl ? (unsigned)d : 0u);
+      if (pm) break;
+    }
+  }
+  if (__any_sync(kFull, timed_out)) {
+    gave_up = true;
+    if (lane == 0) {
+      atomicOr(status, (unsigned)kDevTimeout);
+      st_relaxed_u64(desc + tile, (2ull << 32) | total);
+      if (pos == 31) atomicMax(reinterpret_cast<unsigned long long*>(gdesc + g), (2ull << 32) | total);
+    }
+    return 0u;
+  }
+  if (lane == 0) {
+    const uint64_t inc = (2ull << 32) | (uint32_t)(prefix + total);
+    if (tile != 0) st_relaxed_u64(desc + tile, inc);
+    if (pos == 31) atomicMax(reinterpret_cast<unsigned long long*>(gdesc + g), inc);
+  }
+  return prefix;
+}
+
 // Shape of the row-tile kernel, one CTA per SM.  32-bit values are bound by
 // memory: 9 tiles of 24 KB (192 rows) run 2^28 int32 in 312-321 us, 6 of 32 KB
 // 331, 12 of 16 KB 430 (a prefix per tile becomes the limit).  Compensated
@@ -541,11 +632,27 @@ __global__ void __launch_bounds__(GridCfg<R>::kThreads, 1)
   tile_pipe<C::kNB, C::kNW, 1>(sh->pipe, op, nb, flight, ntiles, ticket, limit, status);
 }
 
-// Short arrays, whose tiles are all resident at once: one tile per CTA in the
-// same three parts, several CTAs per SM, and the prefix gathered by all warps
-// together (every earlier aggregate read once, in one round trip when they
-// are there).  The pipeline serves an SM's tiles one after the other, which
+// Short arrays: one tile per CTA in the same three parts, several CTAs per SM
+// (tiles go by ticket, so that a CTA only waits for tiles of CTAs that run or
+// have run).  The pipeline serves an SM's tiles one after the other, which
 // costs about a microsecond each.
+//
+// The prefix.  32-bit sums take the two-level look-back.  Other values: every
+// earlier aggregate read once, by all warps together, from 33 tiles up only
+// after the tile before has published: until then most are being written, and
+// all CTAs polling all of them made every poll slow.  The wait costs a round
+// trip, and with more tiles than are resident an early reader finds most
+// aggregates there, so it is left out at both ends.  Time until the last
+// prefix, traced on int32 sums of 2^21 / 2^22 / 6 x 10^6 elements: all of them
+// polled at once 8.0 / 8.0 / 10.0 us, after the wait 5.6 / 6.9 / 8.1, look-back
+// 4.3 / 5.2 / 5.9 (fp32: 8.5 / 7.8 / 9.7 and 5.8 / 6.7 / 8.2; a two-level
+// look-back whose group sums are folded in order by the last tile to arrive
+// 7.2 / 8.2 / 9.4).  A call of 2^21 int32 sums, inputs in L2: 9.6 us, 13.8 with
+// all of them polled at once.
+template <class R>
+__host__ __device__ constexpr bool is_sum32() {
+  return std::is_same<R, Plain<AddU>>::value;
+}
 struct GridShortCfg {
   static constexpr int kRows = 256, kNB = 1, kNW = kRows / 32;
   static constexpr uint32_t kTileBytes = kRows * 128;
@@ -555,7 +662,7 @@ template <class R, bool PK>
 __global__ void __launch_bounds__(GridShortCfg::kNW * 32)
     k_scan_grid_short(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtensorMap tout,
                       const uint32_t* __restrict__ in, uint32_t* __restrict__ out, int64_t n, unsigned* ticket,
-                      uint64_t* agg, int excl, uint32_t limit, unsigned* status) {
+                      uint64_t* agg, int64_t ntiles, int excl, int wait, uint32_t limit, unsigned* status) {
   using C = GridShortCfg;
   using V = typename R::V;
   extern __shared__ uint8_t gsr_raw[];
@@ -584,37 +691,70 @@ __global__ void __launch_bounds__(GridShortCfg::kNW * 32)
   }
   op.fold(0, tile);
   __syncthreads();
-  if (warp == 0) op.publish(0, tile);
-  V part = R::ident();
-  bool ok = true;
-  for (int64_t t = tid; t < tile; t += C::kNW * 32) {
-    uint64_t w[2];
-    for (uint32_t polls = 0;; ++polls) {
-      agg_load<R, PK>(agg, t, w);
-      if ((w[0] >> 32) != 0 && (w[1] >> 32) != 0) break;
-      if (polls > limit) {
-        ok = false;
-        break;
-      }
-      __nanosleep(polls > 64 ? 200 : 20);
-    }
-    if (!ok) break;
-    part = R::op(part, agg_value<R>(w));
-  }
-  __syncwarp();
-  part = warp_fold<R>(part);
-  if (lane == 0) s_part[warp] = part;
-  if (__syncthreads_or(!ok)) {
-    if (tid == 0) atomicOr(status, (unsigned)kDevTimeout);
-    return;
-  }
-  if (tid == 0) {
-    V p = R::ident();
+  if constexpr (is_sum32<R>()) {
+    __shared__ int s_bad;
+    if (warp == 0) {
+      unsigned total = 0;
+      if (lane == 0) {
 #pragma unroll
-    for (int k = 0; k < C::kNW; ++k) p = R::op(p, s_part[k]);
-    sh->prefix[0] = p;
+        for (int k = 0; k < C::kNW; ++k) {
+          const unsigned t = sh->wtot[0][k];
+          sh->wtot[0][k] = total;
+          total += t;
+        }
+      }
+      total = __shfl_sync(kFull, total, 0);
+      const int64_t ngroups = (ntiles + 31) / 32;
+      bool gave_up;
+      const unsigned prefix =
+          look_back_sum2(agg, agg + ntiles, agg + ntiles + ngroups, tile, ntiles, total, limit, status, gave_up);
+      if (lane == 0) {
+        sh->prefix[0] = prefix;
+        s_bad = gave_up;
+      }
+    }
+    __syncthreads();
+    if (s_bad) return;
+  } else {
+    if (warp == 0) op.publish(0, tile);
+    V part = R::ident();
+    bool ok = true;
+    auto wait_for = [&](int64_t t, unsigned ns) {  // its aggregate, bounded
+      uint64_t w[2];
+      for (uint32_t polls = 0;; ++polls) {
+        agg_load<R, PK>(agg, t, w);
+        if ((w[0] >> 32) != 0 && (w[1] >> 32) != 0) break;
+        if (polls > limit) {
+          ok = false;
+          break;
+        }
+        __nanosleep(polls > 64 ? 200 : ns);
+      }
+      return agg_value<R>(w);
+    };
+    if (wait) {
+      if (tid == 0 && tile > 0) wait_for(tile - 1, 100);
+      __syncthreads();
+    }
+    for (int64_t t = tid; ok && t < tile; t += C::kNW * 32) {
+      const V a = wait_for(t, 20);
+      part = R::op(part, a);
+    }
+    __syncwarp();
+    part = warp_fold<R>(part);
+    if (lane == 0) s_part[warp] = part;
+    if (__syncthreads_or(!ok)) {
+      if (tid == 0) atomicOr(status, (unsigned)kDevTimeout);
+      return;
+    }
+    if (tid == 0) {
+      V p = R::ident();
+#pragma unroll
+      for (int k = 0; k < C::kNW; ++k) p = R::op(p, s_part[k]);
+      sh->prefix[0] = p;
+    }
+    __syncthreads();
   }
-  __syncthreads();
   op.finish(0, tile);
   __syncthreads();
   if (tid == 0) op.store(0, tile);
@@ -829,30 +969,39 @@ inline ScanWs scan_ws(void* ws, int64_t ntiles) {
   return w;
 }
 
+// Tiles per SM up to which every tile has a CTA of its own (six per SM are
+// resident).  A call with inputs in L2 / in memory, short form | pipeline:
+// int32 sums of 12 / 16.8 / 18 x 10^6 elements 23.9 | 27.1, 33.6 | 35.3, 36.1 |
+// 36.5 us / 28.0 | 28.7, 34.3 | 35.4, 36.5 | 36.7; fp32, which has the dearer
+// prefix, 12 x 10^6 27.7 | 27.2 / 32.2 | 28.7, compensated 26.5 | 28.0 / 30.0 |
+// 28.9.
+template <class R>
+constexpr int grid_short_tiles() {
+  return is_sum32<R>() ? 16 : 8;
+}
+
 // GRID scope over an aligned array of at least one full row.
 template <class R, bool PK>
 static cox_status launch_grid_rows(const uint32_t* in, uint32_t* out, int64_t n, int excl, void* ws, cudaStream_t st) {
   if (!aligned16(ws)) return COX_EINVAL;
-  // Little more than one resident wave of one-tile CTAs (six per SM), or the
-  // pipeline.  2^22 int32 16.9 us against 20.2, 2^23 25.6 against 29.0, 1.26 x
-  // 10^7 31.7 against 30.5, 2^24 37.7 against 35.9; the smallest arrays also
-  // start sooner (10^4: 7.4 against 8.6).
   const int64_t short_tiles = (n + GridShortCfg::kRows * 32 - 1) / (GridShortCfg::kRows * 32);
-  const bool use_short = short_tiles <= (int64_t)8 * sm_count();
+  const bool use_short = short_tiles <= (int64_t)grid_short_tiles<R>() * sm_count();
   using C = GridCfg<R>;
   const int rows = use_short ? GridShortCfg::kRows : C::kRows;
   const int64_t ntiles = use_short ? short_tiles : (n + C::kRows * 32 - 1) / (C::kRows * 32);
   CUtensorMap tin, tout;
   if (!encode_rows32_map(&tin, in, n / 32, rows) || !encode_rows32_map(&tout, out, n / 32, rows))
     return COX_ECUDA;
-  // the ticket, then a zero aggregate per tile (within cox_scan_workspace)
-  if (cudaMemsetAsync(ws, 0, kScanWsHeader + (size_t)ntiles * agg_words<R, PK>() * 8, st) != cudaSuccess)
-    return COX_ECUDA;
+  // the ticket, then a zero aggregate per tile, and the look-back's two words
+  // per group of tiles (within cox_scan_workspace)
+  const size_t words = (size_t)ntiles * agg_words<R, PK>() + (use_short && is_sum32<R>() ? 2 * (size_t)((ntiles + 31) / 32) : 0);
+  if (cudaMemsetAsync(ws, 0, kScanWsHeader + words * 8, st) != cudaSuccess) return COX_ECUDA;
   unsigned* ticket = static_cast<unsigned*>(ws);
   uint64_t* agg = reinterpret_cast<uint64_t*>(static_cast<char*>(ws) + kScanWsHeader);
   if (use_short) {
     k_scan_grid_short<R, PK><<<(unsigned)ntiles, GridShortCfg::kNW * 32, grid_scan_smem<R, GridShortCfg>(1), st>>>(
-        tin, tout, in, out, n, ticket, agg, excl, spin_limit(), device_status_word());
+        tin, tout, in, out, n, ticket, agg, ntiles, excl, ntiles > 32 && ntiles <= (int64_t)6 * sm_count(),
+        spin_limit(), device_status_word());
     return launch_status();
   }
   auto k = k_scan_grid_rows<R, PK>;

@@ -73,20 +73,28 @@ def test_the_pipeline_waits_for_as_many_polls_as_the_limit_says(cox):  # noqa: F
 
 
 @pytest.mark.parametrize("off", [0, 1])
-def test_in_place_through_the_pipeline(cox, off):  # noqa: F811
+def test_compaction_in_place_through_the_pipeline(cox, off):  # noqa: F811
     """A tile is read before anything is written over it."""
     import torch
     k = _keys(_tiles(False) * TILE + 77 + off)[off:]
     want = k[k < THR]
-    ws = torch.empty(cox.cox_scan_workspace(cox.COX_SCOPE_GRID, k.numel()), dtype=torch.uint8, device="cuda")
-    y = torch.empty(k.numel() + off, dtype=torch.int32, device="cuda")[off:]
-    for excl in (0, 1):
-        y.copy_(k)
-        cox.scan(y, exclusive=bool(excl), out=y, workspace=ws)
-        ref = k.long().cumsum(0)
-        if excl:
-            ref -= k.long()
-        assert torch.equal(y, ref.to(torch.int32))
     _, c = cox.ballot_compact(k, THR, out=k)
     assert int(c.item()) == want.numel() and torch.equal(k[:want.numel()], want)
+    assert cox.device_status() == cox.COX_OK
+
+
+@pytest.mark.parametrize("excl", [False, True])
+@pytest.mark.parametrize("delta", [-1, 0, 1])
+@pytest.mark.parametrize("tiles", [1, 33, "most"])
+def test_int_sums_around_the_short_forms_limit(cox, tiles, delta, excl):  # noqa: F811
+    """In place: one tile per CTA up to 16 per SM, with groups of 32 tiles, then the pipeline."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = (16 * sms if tiles == "most" else tiles) * TILE + delta
+    x = torch.randint(-1000, 1000, (n,), dtype=torch.int32, device="cuda")
+    want = x.long().cumsum(0) - (x if excl else 0)
+    room = torch.full((cox.cox_scan_workspace(cox.COX_SCOPE_GRID, n) + 256,), 0xA5, dtype=torch.uint8, device="cuda")
+    cox.scan(x, exclusive=excl, out=x, workspace=room[:-256])
+    assert torch.equal(x, want.to(torch.int32))
+    assert bool((room[-256:] == 0xA5).all())
     assert cox.device_status() == cox.COX_OK
