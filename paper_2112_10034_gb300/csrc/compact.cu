@@ -61,7 +61,9 @@ struct CompactShared {
 // A published count: flag A (desc_missing tells flags 0 and 3 apart from it).
 __device__ __forceinline__ bool count_there(uint64_t d) { return !desc_missing(d); }
 
-template <bool SIGNED, int NB>
+// OFF: the array may begin off a 16-byte boundary (compiled in, the offset costs
+// 0.5% of an aligned array's time in the pipeline).
+template <bool SIGNED, int NB, bool OFF>
 struct CompactOp {
   const uint32_t* keys;
   int64_t n;
@@ -70,23 +72,24 @@ struct CompactOp {
   int64_t* d_count;
   uint64_t* desc;
   int64_t ntiles;
-  int shift;  // words of `keys` past a 16-byte boundary
+  int words_off;  // words of `keys` past a 16-byte boundary
   uint32_t* bufs;
   CompactShared<NB>* sh;
   static constexpr int kWin = 8;  // 32-tile rows per poll of the walk
   int64_t cur = 0, run = 0, base = 0;  // the prefix warp's walk (as AggWalk of the grid scan)
 
-  __device__ uint32_t* buf(int slot) const { return bufs + (size_t)slot * kCompactBuf + shift; }
+  __device__ int shift() const { return OFF ? words_off : 0; }
+  __device__ uint32_t* buf(int slot) const { return bufs + (size_t)slot * kCompactBuf + shift(); }
   __device__ bool bulk(int64_t tile) const {
-    return shift == 0 ? (tile + 1) * kCompactTile <= n : tile > 0 && (tile + 1) * kCompactTile + 4 - shift <= n;
+    return shift() == 0 ? (tile + 1) * kCompactTile <= n : tile > 0 && (tile + 1) * kCompactTile + 4 - shift() <= n;
   }
 
   __device__ void load(int slot, int64_t tile) const {
     uint64_t* bar = sh->pipe.full + slot;
     if (bulk(tile)) {
-      const uint32_t bytes = kCompactTileBytes + (shift ? 16u : 0u);
+      const uint32_t bytes = kCompactTileBytes + (shift() ? 16u : 0u);
       mbar_arrive_expect_tx(bar, bytes);
-      tma_load_1d(buf(slot) - shift, keys + tile * kCompactTile - shift, bytes, bar);
+      tma_load_1d(buf(slot) - shift(), keys + tile * kCompactTile - shift(), bytes, bar);
     } else {
       mbar_arrive(bar);
     }
@@ -96,18 +99,25 @@ struct CompactOp {
     uint32_t* b = buf(slot);
     const int valid = (int)min(kCompactTile, n - tile * kCompactTile);
     if (!bulk(tile)) {
-      // sixteen loads of a lane under way at once: a lone ragged tile is all waiting
-      // (1000 keys 8.2 us a call one after the other, 7.0 so)
       const uint32_t* src = keys + tile * kCompactTile;
+      const int end = min(valid, region + kCompactReg);
+      if constexpr (NB == 1 || OFF) {
+        // sixteen loads of a lane under way at once: a lone ragged tile is all
+        // waiting (1000 keys 8.2 us a call one after the other, 7.0 so), and
+        // everything waits for an unaligned array's first (2^24 keys, d = 0.9:
+        // 40.1 and 37.6)
 #pragma unroll 1
-      for (int i0 = region + lane; i0 < min(valid, region + kCompactReg); i0 += 512) {
-        uint32_t v[16];
+        for (int i0 = region + lane; i0 < end; i0 += 512) {
+          uint32_t v[16];
 #pragma unroll
-        for (int r = 0; r < 16; ++r)
-          if (i0 + 32 * r < valid) v[r] = src[i0 + 32 * r];
+          for (int r = 0; r < 16; ++r)
+            if (i0 + 32 * r < end) v[r] = src[i0 + 32 * r];
 #pragma unroll
-        for (int r = 0; r < 16; ++r)
-          if (i0 + 32 * r < valid) b[i0 + 32 * r] = v[r];
+          for (int r = 0; r < 16; ++r)
+            if (i0 + 32 * r < end) b[i0 + 32 * r] = v[r];
+        }
+      } else {
+        for (int i = region + lane; i < end; i += 32) b[i] = src[i];
       }
       __syncwarp();
     }
@@ -179,14 +189,14 @@ struct CompactOp {
   __device__ void store(int, int64_t) const {}
 };
 
-template <bool SIGNED>
+template <bool SIGNED, bool OFF>
 __global__ void __launch_bounds__(kCompactPipeThreads, 1)
     k_ballot_compact(const uint32_t* __restrict__ keys, int64_t n, int64_t thr, uint32_t* __restrict__ out,
                      int64_t* __restrict__ d_count, unsigned* ticket, uint64_t* desc, int64_t ntiles, int nb,
                      int flight, uint32_t limit, unsigned* status, int shift) {
   extern __shared__ __align__(16) uint32_t smem[];
   auto* sh = reinterpret_cast<CompactShared<kCompactNB>*>(smem + (size_t)nb * kCompactBuf);
-  CompactOp<SIGNED, kCompactNB> op{keys, n, le_rule<SIGNED>(thr), out, d_count, desc, ntiles, shift, smem, sh};
+  CompactOp<SIGNED, kCompactNB, OFF> op{keys, n, le_rule<SIGNED>(thr), out, d_count, desc, ntiles, shift, smem, sh};
   tile_pipe<kCompactNB, kCompactNW, kCompactNG>(sh->pipe, op, nb, flight, ntiles, ticket, limit, status);
 }
 
@@ -202,7 +212,7 @@ __global__ void __launch_bounds__(kCompactThreads, 6)
   __shared__ int64_t s_tile;
   __shared__ uint32_t s_part[kCompactNW];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  CompactOp<SIGNED, 1> op{keys, n, le_rule<SIGNED>(thr), out, d_count, desc, ntiles, shift, smem, sh};
+  CompactOp<SIGNED, 1, true> op{keys, n, le_rule<SIGNED>(thr), out, d_count, desc, ntiles, shift, smem, sh};
   if (tid == 0) {
     mbar_init(sh->pipe.full, 1);
     mbar_init_fence();
@@ -311,8 +321,10 @@ extern "C" cox_status cox_ballot_compact(cox_dtype dt, int width, int block_dim,
                                                                 device_status_word(), shift);
     return launch_status();
   };
-  static int grid_s[kMaxDevices], grid_u[kMaxDevices];  // resident CTAs, per device
-  return dt == COX_I32 ? launch(k_ballot_compact<true>, grid_s) : launch(k_ballot_compact<false>, grid_u);
+  static int grid[4][kMaxDevices];  // resident CTAs, per kernel and device
+  if (shift)
+    return dt == COX_I32 ? launch(k_ballot_compact<true, true>, grid[0]) : launch(k_ballot_compact<false, true>, grid[1]);
+  return dt == COX_I32 ? launch(k_ballot_compact<true, false>, grid[2]) : launch(k_ballot_compact<false, false>, grid[3]);
 }
 
 // ---------------------------------------------------------------------------
