@@ -862,4 +862,11 @@ inline unsigned ring_grid(int64_t nch, int per_warp) {
   return (unsigned)((nch + (int64_t)kRingWarps * per_warp - 1) / ((int64_t)kRingWarps * per_warp));
 }
 
+// Whether nch chunks are more than one but at most `most` for every warp of a
+// row_ring wave (two CTAs of three buffers per SM).
+inline bool ring_few_chunks(int64_t nch, int most) {
+  const int64_t warps = (int64_t)2 * kRingWarps * sm_count();
+  return nch > warps && nch <= most * warps;
+}
+
 }  // namespace cox

@@ -112,13 +112,17 @@ __device__ __forceinline__ void copy_out_padded(const uint32_t* so, uint32_t* __
 // load, and their low words leave in a second pass over the buffer (W = 32
 // 45.0 us in either form; the block sums of reduce_block_rows.cuh lost: 43.4
 // against 47.6).
-template <class R>
-constexpr int tile_stages() {
-  return R::kComp ? kRedStages : 1;
+// A few chunks per resident warp end sooner as one wave for plain reducers too
+// (CTAs start once): 2^24 fp32 with the input in L2, W = 2 / 8, 14.0 / 8.2 us a
+// call against 15.1 / 10.3, 20 x 10^6 20.5 / 10.3 against 20.6 / 12.3; from
+// memory 18.8 / 14.6 either way, 22.4 / 17.0 against 20.8 / 16.6.
+template <int W>
+constexpr int red_wave() {  // chunks per resident warp up to which the wave is taken
+  return W > 2 ? 9 : 7;
 }
 
-template <class R, int W>
-__global__ void __launch_bounds__(kRingWarps * 32, R::kComp ? 2 : 4)
+template <class R, int W, int NS>
+__global__ void __launch_bounds__(kRingWarps * 32, NS > 1 ? 2 : 4)
     k_reduce_tile_rows(const __grid_constant__ CUtensorMap tin, const uint32_t* __restrict__ in,
                        uint32_t* __restrict__ out, float* __restrict__ lo, int64_t n, uint32_t limit,
                        unsigned* status) {
@@ -128,7 +132,7 @@ __global__ void __launch_bounds__(kRingWarps * 32, R::kComp ? 2 : 4)
   const int lane = threadIdx.x & 31;
   const int64_t rows = n / 32;
   const int64_t ntiles = (n + W - 1) / W;
-  row_ring<false, tile_stages<R>()>(&tin, nullptr, rows, (rows + 31) / 32, 32, limit, status,
+  row_ring<false, NS>(&tin, nullptr, rows, (rows + 31) / 32, 32, limit, status,
                                     [&](int64_t c, uint4* buf) {
     V v[32];
 #pragma unroll
@@ -373,6 +377,29 @@ __global__ void __launch_bounds__(1024) k_reduce_grid(const uint32_t* __restrict
 }
 
 // ------------------------------------------------------------------ launch
+// Several buffers: one wave; one buffer: a chunk per warp.
+template <class R, int W, int NS>
+static cox_status launch_tile_rows(const uint32_t* in, uint32_t* out, float* lo, int64_t n, cudaStream_t st) {
+  const int64_t rows = n / 32;
+  CUtensorMap tin;
+  if (!encode_rows32_map(&tin, in, rows, 32)) return COX_ECUDA;
+  auto k = k_reduce_tile_rows<R, W, NS>;
+  constexpr size_t smem = ring_smem(NS);
+  unsigned ctas = ring_grid((rows + 31) / 32, 1);
+  if constexpr (NS > 1) {
+    static int grids[kMaxDevices];  // per device: the resident CTAs
+    int& g = grids[device_index()];
+    if (g == 0) {
+      if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        return COX_ECUDA;
+      g = persistent_grid(k, kRingWarps * 32, smem, 1 << 30);
+    }
+    if (ctas > (unsigned)g) ctas = (unsigned)g;
+  }
+  k<<<ctas, kRingWarps * 32, smem, st>>>(tin, in, out, lo, n, spin_limit(), device_status_word());
+  return launch_status();
+}
+
 template <class R, int W>
 static cox_status launch_reduce(cox_scope scope, const void* d_in, void* d_out, float* d_lo, int64_t n, int B,
                                 unsigned flags, void* ws, size_t ws_bytes, cudaStream_t st) {
@@ -382,23 +409,10 @@ static cox_status launch_reduce(cox_scope scope, const void* d_in, void* d_out, 
   using V = typename R::V;
   if (scope == COX_SCOPE_TILE && n >= 32 && n / 32 < (int64_t(1) << 31) && aligned16(d_in)) {
     // Aligned arrays of at least one full row: the row-per-lane kernel.
-    const int64_t rows = n / 32;
-    CUtensorMap tin;
-    if (!encode_rows32_map(&tin, d_in, rows, 32)) return COX_ECUDA;
-    auto k = k_reduce_tile_rows<R, W>;
-    constexpr size_t smem_rows = ring_smem(tile_stages<R>());
-    static int grids[kMaxDevices];  // per device: the resident CTAs
-    int& gmax_rows = grids[device_index()];
-    if (gmax_rows == 0) {
-      if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_rows) != cudaSuccess)
-        return COX_ECUDA;
-      gmax_rows = persistent_grid(k, kRingWarps * 32, smem_rows, 1 << 30);
-    }
-    const int64_t nch = (rows + 31) / 32;
-    unsigned ctas = ring_grid(nch, 1);
-    if (R::kComp && ctas > (unsigned)gmax_rows) ctas = (unsigned)gmax_rows;
-    k<<<ctas, kRingWarps * 32, smem_rows, st>>>(tin, in, out, d_lo, n, spin_limit(), device_status_word());
-    return launch_status();
+    if constexpr (R::kComp) return launch_tile_rows<R, W, kRedStages>(in, out, d_lo, n, st);
+    else if (ring_few_chunks((n / 32 + 31) / 32, red_wave<W>()))
+      return launch_tile_rows<R, W, kRedStages>(in, out, d_lo, n, st);
+    else return launch_tile_rows<R, W, 1>(in, out, d_lo, n, st);
   }
   if (scope == COX_SCOPE_TILE) {
     auto k = k_reduce_tile<R, W, kRedRows>;

@@ -9,6 +9,8 @@
 // loads, a warp-private shared-memory transpose to one element per lane per
 // row, ROWS independent shuffle chains (instruction-level parallelism), and
 // the inverse transpose to 128-bit stores.
+#include <algorithm>
+
 #include "cox_common.cuh"
 
 namespace cox {
@@ -52,23 +54,28 @@ __global__ void __launch_bounds__(R::kComp ? 256 : 1024) k_tile_scan(const uint3
 // arithmetic: widths 4 / 16 / 32 in 79.9 / 80.0 / 81.7 us, against 80.0 /
 // 87.8 / 94.5 with one chunk, 80.0 / 82.1 / 90.1 with unpacked adds, and 89.2
 // / 94.9 / 89.9 as one persistent wave with unpacked adds.
-template <class R>
-constexpr int rows_stages() {
-  return R::kComp ? 3 : 1;
-}
-template <class R>
-constexpr int rows_chunks() {
-  return R::kComp ? 2 : 1;
+//
+// That is for arrays that stream through memory.  A few chunks per resident
+// warp (two CTAs of three buffers per SM) end sooner as one wave of warps that
+// stride over the array, whose CTAs start once, most of all with the input in
+// L2.  us a call, wave | CTAs from the hardware: plain, width 8, of 2^22 / 2^23
+// / 12 x 10^6 elements 6.2 | 7.1, 8.2 | 10.3, 12.0 | 13.5 (input in memory 8.4
+// | 8.5, 14.3 | 14.0, 18.5 | 18.2; of 16.8 x 10^6 24.3 | 23.1); compensated,
+// width 32, of 2^22 / 2^23 / 2^24 10.3 | 10.3, 12.5 | 14.4, 24.6 | 25.5 (10.6 |
+// 12.3, 14.8 | 17.1, 24.8 | 26.4), width 8 of 2^24 20.8 | 22.6 (24.7 | 24.5).
+template <class R, int W>
+constexpr int rows_wave() {  // chunks per resident warp up to which the wave is taken
+  return !R::kComp ? 5 : W >= 16 ? 9 : 7;
 }
 
-template <class R, int W>
+template <class R, int W, int NS>
 __global__ void __launch_bounds__(kRingWarps * 32, 2)
     k_tile_scan_rows(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtensorMap tout,
                      const uint32_t* __restrict__ in, uint32_t* __restrict__ out, int64_t n, uint32_t limit,
                      unsigned* status) {
   const int lane = threadIdx.x & 31;
   const int64_t rows = n / 32;
-  row_ring<true, rows_stages<R>()>(&tin, &tout, rows, (rows + 31) / 32, 32, limit, status, [&](int64_t, uint4* buf) {
+  row_ring<true, NS>(&tin, &tout, rows, (rows + 31) / 32, 32, limit, status, [&](int64_t, uint4* buf) {
     uint32_t w[32];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {  // unit j of row `lane` sits at unit j ^ (lane & 7)
@@ -97,25 +104,32 @@ __global__ void __launch_bounds__(kRingWarps * 32, 2)
   }
 }
 
-template <class R, int W>
-static cox_status launch_scan_rows(const void* in, void* out, int64_t n, cudaStream_t st) {
-  const int64_t rows = n / 32;
+// One launch over all chunks, `per_warp` of them per warp, or as one wave (0).
+template <class R, int W, int NS>
+static cox_status launch_rows_as(const void* in, void* out, int64_t n, int per_warp, cudaStream_t st) {
+  const int64_t rows = n / 32, nch = (rows + 31) / 32;
   CUtensorMap tin, tout;
   if (!encode_rows32_map(&tin, in, rows, 32) || !encode_rows32_map(&tout, out, rows, 32)) return COX_ECUDA;
-  auto k = k_tile_scan_rows<R, W>;
-  constexpr size_t smem = ring_smem(rows_stages<R>());
-  static bool ready[kMaxDevices];  // per device: the kernel may take its shared memory
-  bool& rd = ready[device_index()];
-  if (!rd) {
+  auto k = k_tile_scan_rows<R, W, NS>;
+  constexpr size_t smem = ring_smem(NS);
+  static int grids[kMaxDevices];  // per device: the resident CTAs
+  int& g = grids[device_index()];
+  if (g == 0) {
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
       return COX_ECUDA;
-    rd = true;
+    g = persistent_grid(k, kRingWarps * 32, smem, 1 << 30);
   }
-  const int64_t nch = (rows + 31) / 32;
-  k<<<ring_grid(nch, rows_chunks<R>()), kRingWarps * 32, smem, st>>>(tin, tout, static_cast<const uint32_t*>(in),
-                                                                     static_cast<uint32_t*>(out), n, spin_limit(),
-                                                                     device_status_word());
+  const unsigned ctas = per_warp ? ring_grid(nch, per_warp) : std::min(ring_grid(nch, 1), (unsigned)g);
+  k<<<ctas, kRingWarps * 32, smem, st>>>(tin, tout, static_cast<const uint32_t*>(in), static_cast<uint32_t*>(out), n,
+                                         spin_limit(), device_status_word());
   return launch_status();
+}
+
+template <class R, int W>
+static cox_status launch_scan_rows(const void* in, void* out, int64_t n, cudaStream_t st) {
+  const bool wave = ring_few_chunks((n / 32 + 31) / 32, rows_wave<R, W>());
+  if constexpr (R::kComp) return launch_rows_as<R, W, 3>(in, out, n, wave ? 0 : 2, st);
+  else return wave ? launch_rows_as<R, W, 3>(in, out, n, 0, st) : launch_rows_as<R, W, 1>(in, out, n, 1, st);
 }
 
 template <class R, int W>

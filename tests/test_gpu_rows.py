@@ -185,3 +185,30 @@ def test_compensated_grid_scan_takes_the_smaller_workspace(cox, n):  # noqa: F81
     err = (out[:n].double() - want).abs() / torch.maximum(want.abs(), 2.0**-24 * x.double().abs().cumsum(0))
     assert float(err.max()) <= 1e-5
     assert bool((ws[need:] == 0xA5).all())
+
+
+@pytest.mark.parametrize("W", [2, 8, 16, 32])
+@pytest.mark.parametrize("per_warp", [1, 5, 7, 9])
+@pytest.mark.parametrize("comp", [0, 1])
+def test_tile_ops_around_the_waves_limits(cox, W, per_warp, comp):  # noqa: F811
+    """A wave of resident warps, or CTAs handed out by the hardware: the same bits as
+    the general kernels (the same values 4 bytes off)."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    edge = 2 * WARPS * sms * per_warp * CHUNK  # chunks of 32 rows per resident warp
+    g = torch.Generator(device="cuda")
+    g.manual_seed(W)
+    off = torch.randn(edge + 66, generator=g, device="cuda")[1:]
+    x = off.clone()
+    for n in (edge, edge + 33):
+        outs = []
+        for src in (x, off):
+            scan, red, lo = poisoned(n, torch.float32), poisoned(-(-n // W), torch.float32), poisoned(-(-n // W), torch.float32)
+            assert cox.cox_tile_scan(o.SUM, o.F32, W, 256, src.data_ptr(), scan.data_ptr(), n, comp, None) == cox.COX_OK
+            assert cox.cox_tile_reduce(o.SUM, o.F32, W, 256, o.TILE, src.data_ptr(), red.data_ptr(), n, comp,
+                                       lo.data_ptr() if comp else None, None, 0, None) == cox.COX_OK
+            outs.append([t.view(torch.int32) for t in (scan, red, lo)])
+        for a, b in zip(*outs):
+            assert torch.equal(a, b)
+            assert bool((a[-64:] == POISON).all())
+    assert cox.device_status() == cox.COX_OK
