@@ -827,11 +827,14 @@ __global__ void __launch_bounds__(1024) k_scan_block(const uint32_t* __restrict_
 // plain and 113 us compensated.
 constexpr int kBlockScanStages = 3, kBlockScanChunks = 2;
 // Smaller arrays are bound by one row's latency, where k_scan_block's warp
-// scan ends sooner: 2^18 elements compensated 4.1 us against 6.2, 2^20 8.2
-// against 6.2; plain 10^3 3.2 against 4.0, 10^5 5.1 (B = 32) against 4.1.
+// scan ends sooner (its blocks of one warp have to take turns).  us in a graph
+// of calls, k_scan_block | rows, plain fp32: B = 256, 2^16 / 2^18 / 2^19
+// elements 1.7 | 2.7, 2.3 | 2.7, 3.4 | 2.7; B = 32, 2^16 / 10^5 / 2^18 2.2 |
+// 2.6, 2.9 | 2.6, 4.1 | 2.6; compensated, B = 256, 2^19 / 2^20 3.9 | 3.9, 5.8 |
+// 3.9.
 template <class R>
-constexpr int64_t block_rows_min() {
-  return R::kComp ? int64_t(1) << 19 : int64_t(1) << 16;
+constexpr int64_t block_rows_min(int block) {
+  return R::kComp ? int64_t(1) << 19 : block < 64 ? int64_t(3) << 15 : int64_t(3) << 17;
 }
 
 template <class R, bool EXCL>
@@ -1030,7 +1033,7 @@ static cox_status launch_scan_scope(cox_scope scope, int block, const void* d_in
   const uint32_t* in = static_cast<const uint32_t*>(d_in);
   uint32_t* out = static_cast<uint32_t*>(d_out);
   if (scope == COX_SCOPE_BLOCK) {
-    if (n >= block_rows_min<R>() && n / 32 < (int64_t(1) << 31) && aligned16(d_in) && aligned16(d_out))
+    if (n >= block_rows_min<R>(block) && n / 32 < (int64_t(1) << 31) && aligned16(d_in) && aligned16(d_out))
       return excl ? launch_block_rows<R, true>(in, out, n, block, st) : launch_block_rows<R, false>(in, out, n, block, st);
     auto k = k_scan_block<R>;
     static int gmax[33];

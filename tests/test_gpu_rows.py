@@ -55,6 +55,24 @@ def test_block_scan_rows_equal_the_general_kernel(cox, B, dt, op, comp, tail):  
     assert torch.equal(y, got[1][:n])
 
 
+@pytest.mark.parametrize("B", [32, 64, 256, 544, 1024])
+@pytest.mark.parametrize("dt,op", [(o.F32, o.SUM), (o.F32, o.MIN), (o.I32, o.SUM)])
+@pytest.mark.parametrize("delta", [-1, 0, 1, 37])
+def test_block_scan_at_the_rows_kernels_smallest_sizes(cox, B, dt, op, delta):  # noqa: F811
+    import torch
+    n = (3 << (15 if B < 64 else 17)) + delta
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n + B)
+    off = torch.randn(n + 1, generator=g, device="cuda").view(torch.int32)[1:]
+    x = off.clone()
+    for excl in (0, 1):
+        got = [poisoned(n, torch.int32) for _ in range(2)]
+        for src, out in zip((x, off), got):
+            assert cox.cox_scan(op, dt, o.BLOCK, B, src.data_ptr(), out.data_ptr(), n, 0, excl, None, 0,
+                                None) == cox.COX_OK
+        assert torch.equal(got[0], got[1]) and bool((got[0][n:] == POISON).all())
+
+
 def _grid_scan(cox, src, n, op, dt, comp, excl):  # noqa: F811
     import torch
     out = poisoned(n, torch.int32)
