@@ -11,7 +11,6 @@
 //   publish the scan of the 8 warp counts; the tile's count;
 //   prefix  the counts of all earlier tiles;
 //   finish  every warp copies its kept keys to out[prefix + offset ..].
-#include <algorithm>
 #include <mutex>
 
 #include "compact_tile.cuh"
@@ -76,7 +75,7 @@ struct CompactOp {
   uint32_t* bufs;
   CompactShared<NB>* sh;
   static constexpr int kWin = 8;  // 32-tile rows per poll of the walk
-  int64_t cur = 0, run = 0, base = 0;  // the prefix warp's walk (as AggWalk of the grid scan)
+  int64_t cur = 0, run = 0;  // the prefix warp's walk: tiles passed, and their counts' sum
 
   __device__ int shift() const { return OFF ? words_off : 0; }
   __device__ uint32_t* buf(int slot) const { return bufs + (size_t)slot * kCompactBuf + shift(); }
@@ -192,12 +191,12 @@ struct CompactOp {
 template <bool SIGNED, bool OFF>
 __global__ void __launch_bounds__(kCompactPipeThreads, 1)
     k_ballot_compact(const uint32_t* __restrict__ keys, int64_t n, int64_t thr, uint32_t* __restrict__ out,
-                     int64_t* __restrict__ d_count, unsigned* ticket, uint64_t* desc, int64_t ntiles, int nb,
-                     int flight, uint32_t limit, unsigned* status, int shift) {
+                     int64_t* __restrict__ d_count, unsigned* ticket, uint64_t* desc, int64_t ntiles,
+                     uint32_t limit, unsigned* status, int shift) {
   extern __shared__ __align__(16) uint32_t smem[];
-  auto* sh = reinterpret_cast<CompactShared<kCompactNB>*>(smem + (size_t)nb * kCompactBuf);
+  auto* sh = reinterpret_cast<CompactShared<kCompactNB>*>(smem + (size_t)kCompactNB * kCompactBuf);
   CompactOp<SIGNED, kCompactNB, OFF> op{keys, n, le_rule<SIGNED>(thr), out, d_count, desc, ntiles, shift, smem, sh};
-  tile_pipe<kCompactNB, kCompactNW, kCompactNG>(sh->pipe, op, nb, flight, ntiles, ticket, limit, status);
+  tile_pipe<kCompactNB, kCompactNW, kCompactNG, kCompactFlight>(sh->pipe, op, ntiles, ticket, limit, status);
 }
 
 // Short arrays, whose tiles are resident at once: one tile per CTA, several
@@ -302,23 +301,17 @@ extern "C" cox_status cox_ballot_compact(cox_dtype dt, int width, int block_dim,
     };
     return dt == COX_I32 ? go(k_ballot_compact_short<true>) : go(k_ballot_compact_short<false>);
   }
-  auto smem = [](int nb) { return (size_t)nb * kCompactBuf * 4 + sizeof(CompactShared<kCompactNB>); };
+  constexpr size_t smem = (size_t)kCompactNB * kCompactBuf * 4 + sizeof(CompactShared<kCompactNB>);
   auto launch = [&](auto kern, int* grid) {
     int& g = grid[device_index()];
     if (g == 0) {
-      if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem(kCompactNB)) !=
-          cudaSuccess)
+      if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return COX_ECUDA;
-      g = persistent_grid(kern, kCompactPipeThreads, smem(kCompactNB), 1 << 30);
+      g = persistent_grid(kern, kCompactPipeThreads, smem, 1 << 30);
     }
-    // as many buffers as give every CTA work, in whole rounds of the groups
-    const int64_t ctas = ntiles < g ? ntiles : g;
-    int nb = (int)std::min<int64_t>(kCompactNB, (ntiles + ctas - 1) / ctas);
-    if (nb > kCompactNG) nb = (nb + kCompactNG - 1) / kCompactNG * kCompactNG;
-    const int flight = ntiles <= ctas * nb ? nb : kCompactFlight;
-    kern<<<(unsigned)ctas, kCompactPipeThreads, smem(nb), st>>>(keys, n, threshold, outp, d_count, ticket, desc,
-                                                                ntiles, nb, flight, spin_limit(),
-                                                                device_status_word(), shift);
+    // (one CTA per SM, and more tiles than all of them have buffers)
+    kern<<<(unsigned)g, kCompactPipeThreads, smem, st>>>(keys, n, threshold, outp, d_count, ticket, desc, ntiles,
+                                                         spin_limit(), device_status_word(), shift);
     return launch_status();
   };
   static int grid[4][kMaxDevices];  // resident CTAs, per kernel and device

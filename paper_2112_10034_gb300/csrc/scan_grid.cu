@@ -18,7 +18,6 @@
 // and its inclusive prefix in separate slots, each written before its flag
 // (release store) and read after it (acquire load), so a reader never sees a
 // value from the wrong stage.
-#include <algorithm>
 #include <type_traits>
 
 #include "cox_common.cuh"
@@ -497,8 +496,8 @@ struct GridScanShared {
   typename R::V prefix[C::kNB];
 };
 template <class R, class C>
-constexpr size_t grid_scan_smem(int nb) {
-  return 1024 + (size_t)nb * C::kTileBytes + sizeof(GridScanShared<R, C>);
+constexpr size_t grid_scan_smem() {
+  return 1024 + (size_t)C::kNB * C::kTileBytes + sizeof(GridScanShared<R, C>);
 }
 
 template <class R, class C, bool PK>
@@ -621,15 +620,14 @@ template <class R, bool PK>
 __global__ void __launch_bounds__(GridCfg<R>::kThreads, 1)
     k_scan_grid_rows(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtensorMap tout,
                      const uint32_t* __restrict__ in, uint32_t* __restrict__ out, int64_t n, unsigned* ticket,
-                     uint64_t* agg, int64_t ntiles, int excl, int nb, int flight, uint32_t limit,
-                     unsigned* status) {
+                     uint64_t* agg, int64_t ntiles, int excl, uint32_t limit, unsigned* status) {
   using C = GridCfg<R>;
   extern __shared__ uint8_t gsr_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(gsr_raw) + 1023) & ~uintptr_t(1023));
-  GridScanShared<R, C>* sh = reinterpret_cast<GridScanShared<R, C>*>(base + (size_t)nb * C::kTileBytes);
+  GridScanShared<R, C>* sh = reinterpret_cast<GridScanShared<R, C>*>(base + (size_t)C::kNB * C::kTileBytes);
   GridScanOp<R, C, PK> op{&tin, &tout, in, out, n, n / 32, agg, excl, reinterpret_cast<uint4*>(base), sh, 0,
                    R::ident()};
-  tile_pipe<C::kNB, C::kNW, 1>(sh->pipe, op, nb, flight, ntiles, ticket, limit, status);
+  tile_pipe<C::kNB, C::kNW, 1, C::kFlight>(sh->pipe, op, ntiles, ticket, limit, status);
 }
 
 // Short arrays: one tile per CTA in the same three parts, several CTAs per SM
@@ -1002,7 +1000,7 @@ static cox_status launch_grid_rows(const uint32_t* in, uint32_t* out, int64_t n,
   unsigned* ticket = static_cast<unsigned*>(ws);
   uint64_t* agg = reinterpret_cast<uint64_t*>(static_cast<char*>(ws) + kScanWsHeader);
   if (use_short) {
-    k_scan_grid_short<R, PK><<<(unsigned)ntiles, GridShortCfg::kNW * 32, grid_scan_smem<R, GridShortCfg>(1), st>>>(
+    k_scan_grid_short<R, PK><<<(unsigned)ntiles, GridShortCfg::kNW * 32, grid_scan_smem<R, GridShortCfg>(), st>>>(
         tin, tout, in, out, n, ticket, agg, ntiles, excl, ntiles > 32 && ntiles <= (int64_t)6 * sm_count(),
         spin_limit(), device_status_word());
     return launch_status();
@@ -1011,19 +1009,14 @@ static cox_status launch_grid_rows(const uint32_t* in, uint32_t* out, int64_t n,
   static int grid[kMaxDevices];  // resident CTAs, per device
   int& g = grid[device_index()];
   if (g == 0) {
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)grid_scan_smem<R, C>(C::kNB)) !=
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)grid_scan_smem<R, C>()) !=
         cudaSuccess)
       return COX_ECUDA;
-    g = persistent_grid(k, C::kThreads, grid_scan_smem<R, C>(C::kNB), 1 << 30);
+    g = persistent_grid(k, C::kThreads, grid_scan_smem<R, C>(), 1 << 30);
   }
-  // as many buffers as give every CTA work: an array's tiles spread over the
-  // CTAs instead of queueing in the first ones; one that fits the buffers is
-  // loaded all at once
-  const int64_t ctas = ntiles < g ? ntiles : g;
-  const int nb = (int)std::min<int64_t>(C::kNB, (ntiles + ctas - 1) / ctas);
-  const int flight = ntiles <= ctas * nb ? nb : C::kFlight;
-  k<<<(unsigned)ctas, C::kThreads, grid_scan_smem<R, C>(nb), st>>>(tin, tout, in, out, n, ticket, agg, ntiles, excl,
-                                                                   nb, flight, spin_limit(), device_status_word());
+  // (one CTA per SM, and more tiles than all of them have buffers)
+  k<<<(unsigned)g, C::kThreads, grid_scan_smem<R, C>(), st>>>(tin, tout, in, out, n, ticket, agg, ntiles, excl,
+                                                              spin_limit(), device_status_word());
   return launch_status();
 }
 

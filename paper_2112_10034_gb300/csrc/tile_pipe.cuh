@@ -82,10 +82,12 @@ struct PipePos {
   __device__ uint32_t parity() const { return round & 1u; }
 };
 
-// Runs the pipeline on a CTA of NG * NW + 3 warps, nb <= NB of the buffers in
-// use and at most `flight` loads in flight.  The workers are NG groups of NW
-// warps, group g taking every NG-th of the CTA's tiles from its g-th on.  `op` provides, with `slot` the tile's
-// buffer:
+// Runs the pipeline on a CTA of NG * NW + 3 warps with FL loads in flight.  The
+// workers are NG groups of NW warps, group g taking every NG-th of the CTA's
+// tiles from its g-th on: NG divides NB, so that a slot's tiles belong to one
+// group, which has finished the slot's last tile before it asks for the next (a
+// parity can only be told from the one before).  `op` provides, with `slot` the
+// tile's buffer:
 //   load(slot, tile)     one thread: starts the copies that complete full[slot]
 //   fold(slot, tile)     each worker warp: its part of the tile's aggregate
 //   publish(slot, tile)  the last worker warp to fold it
@@ -94,15 +96,11 @@ struct PipePos {
 //   finish(slot, tile)   each worker warp: its part of the results
 //   store(slot, tile)    one thread: copies out of the buffer; returns when
 //                        they have read it
-template <int NB, int NW, int NG, class Op>
-__device__ __forceinline__ void tile_pipe(PipeShared<NB>& ps, Op& op, int nb, int flight, int64_t ntiles,
-                                          unsigned* ticket, uint32_t limit, unsigned* status) {
+template <int NB, int NW, int NG, int FL, class Op>
+__device__ __forceinline__ void tile_pipe(PipeShared<NB>& ps, Op& op, int64_t ntiles, unsigned* ticket,
+                                          uint32_t limit, unsigned* status) {
+  static_assert(NB % NG == 0 && FL <= NB);
   const int warp = threadIdx.x >> 5, lane = lane_id();
-  // Worker groups in use: a divisor of nb, so that a slot's tiles belong to
-  // one group, which has finished the slot's last tile before it asks for the
-  // next (a parity can only be told from the one before).
-  int ng = min(NG, nb);
-  while (nb % ng) --ng;
   if (threadIdx.x == 0) {
     for (int b = 0; b < NB; ++b) {
       mbar_init(ps.full + b, 1);
@@ -123,21 +121,21 @@ __device__ __forceinline__ void tile_pipe(PipeShared<NB>& ps, Op& op, int nb, in
     }
   };
   if (warp == NG * NW) {  // ------------------------------------------- loader
-    PipePos at, ahead;  // the next tile; the one `flight` before it
+    PipePos at, ahead;  // the next tile; the one FL before it
     bool ok = true;
     int64_t k = 0;
     int marked = 0;  // slots that have been told of the end
     unsigned t = 0;
     for (;; ++k) {
-      if (k >= nb) ok = pipe_wait(ps, ps.free + at.slot, at.parity() ^ 1u, limit);
-      if (ok && k >= flight) {
+      if (k >= NB) ok = pipe_wait(ps, ps.free + at.slot, at.parity() ^ 1u, limit);
+      if (ok && k >= FL) {
         ok = pipe_wait(ps, ps.full + ahead.slot, ahead.parity(), limit);
-        ahead.next(nb);
+        ahead.next(NB);
       }
       if (!ok) break;
-      // the first `flight` tiles are asked for together: one round trip
-      if (k == 0 || k >= flight) {
-        if (lane == 0) t = atomicAdd(ticket, k == 0 ? (unsigned)flight : 1u);
+      // the first FL tiles are asked for together: one round trip
+      if (k == 0 || k >= FL) {
+        if (lane == 0) t = atomicAdd(ticket, k == 0 ? (unsigned)FL : 1u);
       } else {
         ++t;
       }
@@ -153,11 +151,11 @@ __device__ __forceinline__ void tile_pipe(PipeShared<NB>& ps, Op& op, int nb, in
         marked = 1;
         break;
       }
-      at.next(nb);
+      at.next(NB);
     }
-    for (int i = 1; ok && i < ng; ++i) {  // the other groups hear of the end on the slots after
-      at.next(nb);
-      if (k + i >= nb) ok = pipe_wait(ps, ps.free + at.slot, at.parity() ^ 1u, limit);
+    for (int i = 1; ok && i < NG; ++i) {  // the other groups hear of the end on the slots after
+      at.next(NB);
+      if (k + i >= NB) ok = pipe_wait(ps, ps.free + at.slot, at.parity() ^ 1u, limit);
       if (ok && lane == 0) {
         ps.tile[at.slot] = -1;
         mbar_arrive(ps.full + at.slot);
@@ -166,13 +164,13 @@ __device__ __forceinline__ void tile_pipe(PipeShared<NB>& ps, Op& op, int nb, in
     }
     if (!ok) give_up();
     if (lane == 0)  // whatever becomes of the CTA, its copies in flight land before it ends
-      for (int64_t i = k + marked > nb ? k + marked - nb : 0; i < k; ++i)
-        mbar_drain(ps.full + (int)(i % nb), (uint32_t)((i / nb) & 1));
+      for (int64_t i = k + marked > NB ? k + marked - NB : 0; i < k; ++i)
+        mbar_drain(ps.full + (int)(i % NB), (uint32_t)((i / NB) & 1));
     __syncwarp();
     return;
   }
   if (warp == NG * NW + 2) {  // --------------------------------------- prefix
-    for (PipePos at;; at.next(nb)) {
+    for (PipePos at;; at.next(NB)) {
       if (!pipe_wait(ps, ps.full + at.slot, at.parity(), limit)) break;
       const int64_t tile = ps.tile[at.slot];
       if (tile < 0) return;
@@ -186,7 +184,7 @@ __device__ __forceinline__ void tile_pipe(PipeShared<NB>& ps, Op& op, int nb, in
     return;
   }
   if (warp == NG * NW + 1) {  // ---------------------------------------- store
-    for (PipePos at;; at.next(nb)) {
+    for (PipePos at;; at.next(NB)) {
       if (!pipe_wait(ps, ps.full + at.slot, at.parity(), limit)) break;
       const int64_t tile = ps.tile[at.slot];
       if (tile < 0) return;
@@ -202,17 +200,16 @@ __device__ __forceinline__ void tile_pipe(PipeShared<NB>& ps, Op& op, int nb, in
   }
   // ---------------------------------------------------------- workers
   const int group = warp / NW;
-  if (group >= ng) return;
   PipePos f, p;  // the next tile to fold, to finish
   for (int i = 0; i < group; ++i) {
-    f.next(nb);
-    p.next(nb);
+    f.next(NB);
+    p.next(NB);
   }
   int held = 0;  // slots from p to f
   bool ended = false;
   uint32_t spin = 0;
   for (;;) {
-    if (!ended && held < nb && __all_sync(kFull, mbar_test(ps.full + f.slot, f.parity()))) {
+    if (!ended && held < NB && __all_sync(kFull, mbar_test(ps.full + f.slot, f.parity()))) {
       const int64_t tile = ps.tile[f.slot];
       spin = 0;
       if (tile < 0) {
@@ -235,8 +232,8 @@ __device__ __forceinline__ void tile_pipe(PipeShared<NB>& ps, Op& op, int nb, in
           mbar_arrive(ps.folded + f.slot);
         }
       }
-      held += ng;
-      for (int i = 0; i < ng; ++i) f.next(nb);
+      held += NG;
+      for (int i = 0; i < NG; ++i) f.next(NB);
       continue;
     }
     if (held) {
@@ -245,8 +242,8 @@ __device__ __forceinline__ void tile_pipe(PipeShared<NB>& ps, Op& op, int nb, in
         op.finish(p.slot, ps.tile[p.slot]);
         __syncwarp();
         if (lane == 0) mbar_arrive(ps.done + p.slot);
-        held -= ng;
-        for (int i = 0; i < ng; ++i) p.next(nb);
+        held -= NG;
+        for (int i = 0; i < NG; ++i) p.next(NB);
         continue;
       }
     } else if (ended) {
