@@ -162,7 +162,8 @@ cox_status cox_tile_scan(cox_op op, cox_dtype dt, int width, int block_dim, cons
  * 6144 or 8192 elements by TMA; other layouts: 16384, 8192 compensated): in a
  * tile every warp scans its rows of 32 elements, carries row totals across its
  * rows, the warp totals are scanned, the tile publishes its aggregate, and its
- * prefix -- the fold of all earlier tiles' aggregates -- is added.
+ * prefix -- the fold of all earlier tiles' aggregates -- is added.  (Short
+ * arrays of 32-bit integers find the sums of earlier tiles by a look-back.)
  *   d_out[i] = x[s] op ... op x[i] (inclusive) or x[s] op ... op x[i-1] with
  *   the identity at i = s (exclusive), s = the first index of i's block
  *   (BLOCK) or 0 (GRID).
@@ -170,6 +171,10 @@ cox_status cox_tile_scan(cox_op op, cox_dtype dt, int width, int block_dim, cons
  *   exclusive: 0 or 1.
  *   d_workspace: GRID only, cox_scan_workspace() bytes, 16-byte aligned,
  *   zeroed by the call (cudaMemsetAsync).  Not shared across concurrent calls.
+ *   Compensated sums of 16-byte aligned arrays also take 256 + (4 t rounded up
+ *   to 256) + 16 t + 24 ceil(t / 32) bytes, t = ceil(n / 16384): a tile's
+ *   aggregate then passes on with its error word rounded to 21 mantissa bits
+ *   (about 2^-46 of the sum).
  * Integer results are exact.  GRID fp32 results take each tile's prefix in the
  * order in which the earlier aggregates were found, so their last bits may
  * differ from run to run (within the stated tolerance).  BLOCK results are
@@ -314,8 +319,8 @@ size_t cox_integral_image_workspace(int64_t batch, int64_t height, int64_t width
  *   d_count: one int64 on the device, receives the number kept.
  *   d_workspace: at least cox_ballot_compact_workspace(n, block_dim) bytes,
  *   16-byte aligned; the call zeroes it first (a cudaMemsetAsync on `stream`)
- *   unless flags has COX_F_WS_READY, in which case the caller guarantees those
- *   bytes are zero.  Not shared across concurrent calls.
+ *   unless flags has COX_F_WS_READY, in which case the caller guarantees that
+ *   all of those bytes (a ticket, descriptors) are zero.  Not shared across concurrent calls.
  *   flags: 0 or COX_F_WS_READY.
  * Tiles of 8192 keys (whatever block_dim: the result does not depend on the
  * block size, which is only validated) are handed to the CTAs by an atomic

@@ -4,10 +4,8 @@
 // ragged tile) and go through the tile pipeline (tile_pipe.cuh; short arrays:
 // one tile per CTA).  In a tile, by eight warps:
 //   fold    every warp compacts its 1024 keys in place in one pass
-//           (compact_tile.cuh): per chunk of 128 keys, b =
-//           __ballot_sync(keep) for each of a lane's four key slots, rank =
-//           kept keys before the chunk + popc(b & lanemask_lt) over the slots
-//           + kept keys before it in the lane;
+//           (compact_tile.cuh): per row of 32 keys, b = __ballot_sync(keep),
+//           rank = kept keys of earlier rows + popc(b & lanemask_lt);
 //   publish the scan of the 8 warp counts; the tile's count;
 //   prefix  the counts of all earlier tiles;
 //   finish  every warp copies its kept keys to out[prefix + offset ..].
@@ -28,13 +26,13 @@ constexpr uint32_t kCompactTileBytes = (uint32_t)kCompactTile * 4;
 // boundary before the tile to the one after it (words of the neighbouring
 // tiles, never beyond the array) and its tile sits `shift` words into the
 // buffer.  The first tile, and one whose copy would pass the array's end, are
-// loaded word by word.  2^28 keys 4 bytes off, d = 0.1 / 0.5 / 0.9: 256 / 291 / 331 us;
-// loaded word by word in fold, which every later tile waits for, 703 / 751 /
+// loaded word by word.  2^28 keys 4 bytes off, d = 0.1 / 0.5 / 0.9: 256 / 291 /
+// 331 us; all tiles loaded word by word in fold, which every later tile waits for, 703 / 751 /
 // 789 (577 / 649 / 715 by the cooperative kernel before the pipeline).
 constexpr int kCompactBuf = (int)kCompactTile + 4;
 // Shape of the pipeline, one CTA per SM: six tiles, two groups of eight worker
-// warps, three loads in flight.  2^28 keys at d = 0.1 / 0.5 / 0.9: 249 / 283 /
-// 323 us (4740 / 5700 / 6310 GB/s); one group 344 / 367 / 394, three 252 / 283
+// warps, three loads in flight.  2^28 keys at d = 0.1 / 0.5 / 0.9: 246 / 281 /
+// 322 us (4800 / 5730 / 6340 GB/s); one group 344 / 367 / 394, three 252 / 283
 // / 322 (the workers' passes over the keys, then the tile's way through shared
 // memory, bound it).  The cooperative kernel before it, two tiles per CTA and a
 // look-back per tile, ran 271 / 326 / 372 us, with this tile body 273 / 327 /
@@ -42,9 +40,11 @@ constexpr int kCompactBuf = (int)kCompactTile + 4;
 constexpr int kCompactNB = 6;      // tiles in shared memory
 constexpr int kCompactNG = 2;      // groups of eight worker warps
 constexpr int kCompactFlight = 3;  // loads in flight
-// Up to this many tiles per SM every tile has a CTA of its own (six fit).
-// 10^6 keys at d = 0.5 8.3 us against 10.3 through the pipeline, 2^22 13.8
-// against 17.9, 2^23 22.4 against 22.0, 2^24 32.3 against 30.2.
+// Up to this many tiles per SM every tile has a CTA of its own (six fit).  us a
+// call at d = 0.5, inputs in L2 (in memory), one tile per CTA | pipeline | the
+// cooperative kernel: 10^6 keys 8.2 | 11.2 | 8.3 (9.1 | 12.4 | 9.1), 2^22 13.4 |
+// 15.4 | 13.5 (15.4 | 17.3 | 15.9), 2^23 21.5 | 18.6 | 17.5 (22.1 | 19.8 | 20.2),
+// 2^24 32.2 | 26.8 | 25.7 (32.5 | 29.2 | 29.1).
 constexpr int kCompactShortTiles = 6;
 constexpr int kCompactPipeThreads = (kCompactNG * kCompactNW + 3) * 32;
 

@@ -64,7 +64,8 @@ constexpr uint64_t kGroupSumMask = kGroupArrive - 1;
 __host__ __device__ inline int64_t compact_groups(int64_t ntiles) {
   return (ntiles + (1 << kGroupShift) - 1) >> kGroupShift;
 }
-// Workspace bytes of a compaction over ntiles tiles: a header (reserved), tile
+// Workspace bytes of a compaction over ntiles tiles: a header (its first
+// word the ticket by which tiles are handed out, in cox_ballot_compact), tile
 // descriptors, group descriptors and group accumulators.
 __host__ __device__ inline size_t compact_ws_bytes(int64_t ntiles) {
   return kCompactWsHeader + (size_t)ntiles * 8 + (size_t)compact_groups(ntiles) * 16;

@@ -570,9 +570,9 @@ __device__ __forceinline__ void mbar_drain(uint64_t* bar, uint32_t parity) {
 // within `limit` polls records kDevTimeout, gives the copies in flight a
 // bounded wait and ends the warp's loop.  CTAs are kRingWarps warps.
 //
-// Launches give every warp one or two chunks (ring_grid) and let the hardware
-// hand out CTAs, instead of one resident wave whose warps stride over the
-// array: SMs do not reach memory at equal rates, so equal shares end in a
+// Launches over many chunks give every warp one or two (ring_grid) and let the
+// hardware hand out CTAs, instead of one resident wave whose warps stride over
+// the array (the better one for a few chunks per warp, ring_few_chunks): SMs do not reach memory at equal rates, so equal shares end in a
 // tail of the slower ones.  2^26 elements copied through this ring (GB300):
 // one wave of 304 CTAs 88.9 us (6037 GB/s), 8 / 4 / 2 / 1 chunks per warp
 // 84.0 / 81.5 / 80.3 / 79.6 us (6747 GB/s, the device's copy rate).

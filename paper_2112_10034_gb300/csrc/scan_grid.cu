@@ -463,11 +463,12 @@ __global__ void __launch_bounds__(256) k_scan_grid(const uint32_t* __restrict__ 
 }
 
 // GRID scope over aligned arrays of at least one full row, through tile_pipe:
-// a tile of 256 rows of 32 elements arrives by one 2D TMA box with 128-byte
-// swizzle; lane t of worker w owns row 32 w + t of the tile.  fold: each lane
-// folds its row, a shuffle scan over the warp's rows gives every row's
-// exclusive prefix in the warp; publish: the scan of the 8 warp totals, the
-// tile's aggregate; prefix: the walk over the earlier tiles' aggregates;
+// a tile of 192 rows of 32 elements (compensated pairs and short arrays: 256)
+// arrives by one 2D TMA box with 128-byte swizzle; lane t of worker w owns row
+// 32 w + t of the tile.  fold: each lane folds its row, a shuffle scan over the
+// warp's rows gives every row's exclusive prefix in the warp; publish: the scan
+// of the warp totals (one per 32 rows), the tile's aggregate; prefix: the walk
+// over the earlier tiles' aggregates;
 // finish: re-reads the row, carrying prefix op value into each element (in
 // place), before one TMA store.  Sums are folded left to right within a row,
 // so fp32 results differ from the shuffle form in their last bits

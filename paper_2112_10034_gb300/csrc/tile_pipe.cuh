@@ -23,8 +23,10 @@
 // tile only once that tile is published: most earlier ones are by then, and
 // walking as soon as the tile's number is known, at the frontier all the time,
 // measured 344 us against 331 on 2^28 int32.  Publishing is one
-// store, without atomics, group words or inclusive prefixes, and a running
-// prefix is always the same sequence of combines.
+// store (compaction: one atomicMax, which leaves a withheld word alone), without
+// group words or inclusive prefixes.  A poll folds as many aggregates as are
+// there, so the order in which fp32 sums are combined, and with it their last
+// bits, may differ from run to run.
 //
 // Every wait ends: tickets are only given to running CTAs, and no tile's
 // publishing waits for a prefix (its buffer is free when it gets its ticket,
@@ -69,7 +71,7 @@ __device__ __forceinline__ bool pipe_wait(PipeShared<NB>& ps, uint64_t* bar, uin
   return false;
 }
 
-// A position in the ring of nb buffers and the parity of its round.
+// A position in a ring of nb buffers and the parity of its round.
 struct PipePos {
   int slot = 0;
   uint32_t round = 0;
