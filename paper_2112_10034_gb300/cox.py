@@ -283,13 +283,8 @@ def _dtype_code(x, unsigned: bool = False) -> int:
     raise TypeError(f"32-bit int or float tensor required, got {x.dtype}")
 
 
-def _workspace(workspace, need, dev):
-    """(tensor, its own size in bytes): the caller's workspace, else a new one of `need` bytes (0: none)."""
-    if workspace is None:
-        if not need:
-            return None, 0
-        workspace = _torch().empty(need, dtype=_torch().uint8, device=dev)
-    return workspace, workspace.numel() * workspace.element_size()
+def _bytes(t) -> int:
+    return t.numel() * t.element_size()
 
 
 def _dev_tensor(x):
@@ -332,7 +327,11 @@ def tile_reduce(x, op: int = COX_SUM, width: int = 32, block_dim: int = 256, sco
         out = t.empty(m, dtype=x.dtype, device=x.device)
     lo = t.zeros(m, dtype=t.float32, device=x.device) if with_lo else None
     flags = (COX_F_COMPENSATED if compensated else 0) | (COX_F_FP64_COMBINE if fp64_combine else 0)
-    workspace, ws_bytes = _workspace(workspace, cox_tile_reduce_workspace(scope, n, block_dim), x.device)
+    ws_bytes = cox_tile_reduce_workspace(scope, n, block_dim)
+    if workspace is not None:
+        ws_bytes = _bytes(workspace)  # its own size, not the one it should have
+    elif ws_bytes:
+        workspace = t.empty(ws_bytes, dtype=t.uint8, device=x.device)
     _check(cox_tile_reduce(op, _dtype_code(x, unsigned), width, block_dim, scope, x.data_ptr(), out.data_ptr(), n,
                            flags, lo.data_ptr() if lo is not None else None,
                            workspace.data_ptr() if workspace is not None else None, ws_bytes,
@@ -359,7 +358,11 @@ def scan(x, op: int = COX_SUM, scope: int = COX_SCOPE_GRID, block_dim: int = 256
     x = _dev_tensor(x)
     if out is None:
         out = t.empty_like(x)
-    workspace, ws_bytes = _workspace(workspace, cox_scan_workspace(scope, x.numel()), x.device)
+    ws_bytes = cox_scan_workspace(scope, x.numel())
+    if workspace is not None:
+        ws_bytes = _bytes(workspace)  # its own size, not the one it should have
+    elif ws_bytes:
+        workspace = t.empty(ws_bytes, dtype=t.uint8, device=x.device)
     _check(cox_scan(op, _dtype_code(x, unsigned), scope, block_dim, x.data_ptr(), out.data_ptr(), x.numel(),
                     COX_F_COMPENSATED if compensated else 0, 1 if exclusive else 0,
                     workspace.data_ptr() if workspace is not None else None, ws_bytes, _stream(x.device)),
@@ -373,7 +376,11 @@ def grid_broadcast(x, op: int = COX_GRID_SUB_MIN, unsigned: bool = False, out=No
     x = _dev_tensor(x)
     if out is None:
         out = t.empty_like(x)
-    workspace, ws_bytes = _workspace(workspace, cox_grid_broadcast_workspace(x.numel()), x.device)
+    ws_bytes = cox_grid_broadcast_workspace(x.numel())
+    if workspace is not None:
+        ws_bytes = _bytes(workspace)
+    else:
+        workspace = t.empty(ws_bytes, dtype=t.uint8, device=x.device)
     _check(cox_grid_broadcast(op, _dtype_code(x, unsigned), x.data_ptr(), out.data_ptr(), x.numel(),
                               workspace.data_ptr(), ws_bytes, _stream(x.device)), "cox_grid_broadcast")
     return out
