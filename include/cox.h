@@ -536,7 +536,7 @@ typedef struct {
   int64_t batches;      /* persistent launches so far */
   int64_t max_batch;    /* most requests in one launch */
   size_t budget_bytes;  /* admission budget */
-  size_t used_bytes;    /* held by admitted, unreleased requests */
+  size_t used_bytes;    /* held by admitted requests until released and read out (cox_server_read) */
   size_t peak_bytes;    /* most ever held */
   int64_t queued;       /* submitted, waiting for admission */
   double wait_s;        /* summed over completed requests: submit to launch (queueing and batching) */

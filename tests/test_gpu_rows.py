@@ -230,3 +230,53 @@ def test_tile_ops_around_the_waves_limits(cox, W, per_warp, comp):  # noqa: F811
             assert torch.equal(a, b)
             assert bool((a[-64:] == POISON).all())
     assert cox.device_status() == cox.COX_OK
+
+
+@pytest.mark.parametrize("kind", ["inf", "nan", "zeros", "tiny", "huge"])
+def test_special_values_as_in_the_general_kernels(cox, kind):  # noqa: F811
+    """Infinities, NaN, signed zeros, denormals and overflow: aligned arrays (rows kernels, short form and pipeline)
+    give what the same values 4 bytes off give, NaN for NaN."""
+    import torch
+
+    def same(a, b):
+        fa, fb = a.view(torch.float32), b.view(torch.float32)
+        return bool(((a == b) | (fa.isnan() & fb.isnan())).all())
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    for n in (600_003, 10 * sms * SHORT_TILE + 5):
+        g = torch.Generator(device="cuda")
+        g.manual_seed(n)
+        off = torch.randn(n + 1, generator=g, device="cuda")[1:]
+        idx = torch.randint(0, n, (n // 5000,), generator=g, device="cuda")
+        if kind == "inf":
+            off[idx], off[idx // 2] = float("inf"), -float("inf")
+        elif kind == "nan":
+            off[idx], off[0] = float("nan"), float("nan")
+        elif kind == "zeros":
+            off.zero_()
+            off[idx] = -0.0
+            off[:2000] = -0.0
+        else:
+            off.mul_(1e-40 if kind == "tiny" else 3e38)
+        x = off.clone()
+        ws = torch.empty(cox.cox_scan_workspace(o.GRID, n), dtype=torch.uint8, device="cuda")
+        for op, comp in ((o.SUM, 0), (o.SUM, 1), (o.MIN, 0), (o.MAX, 0)):
+            outs = {}
+            for at, src in (("on", x), ("off", off)):
+                for B in (32, 256):
+                    for excl in (0, 1):
+                        out = poisoned(n, torch.int32)
+                        assert cox.cox_scan(op, o.F32, o.BLOCK, B, src.data_ptr(), out.data_ptr(), n, comp, excl, None, 0,
+                                            None) == cox.COX_OK
+                        outs[at, B, excl] = out[:n]
+                for W in (2, 32):
+                    out = poisoned(n, torch.int32)
+                    assert cox.cox_tile_scan(op, o.F32, W, 256, src.data_ptr(), out.data_ptr(), n, comp, None) == cox.COX_OK
+                    outs[at, W] = out[:n]
+                if op != o.SUM:  # (sums are folded in another order)
+                    out = poisoned(n, torch.int32)
+                    assert cox.cox_scan(op, o.F32, o.GRID, 256, src.data_ptr(), out.data_ptr(), n, 0, 0, ws.data_ptr(),
+                                        ws.numel(), None) == cox.COX_OK
+                    outs[at, "grid"] = out[:n]
+            for key in [k for k in outs if k[0] == "on"]:
+                assert same(outs[key], outs[("off",) + key[1:]]), (kind, n, op, comp, key)
+    assert cox.device_status() == cox.COX_OK
